@@ -57,17 +57,18 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.82 MB read + 0.29 MB written for
+# small case at 16 CTAs (1x1024^2: 5.50 MB read + 0.27 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.82
-TRAFFIC_SRC_SHA = "e10c941e99c22be48bf826ed2ee2ac989cf61d75567d02f7f1d9470621dcf631"
+TRAFFIC_B_PER_PX = 5.50
+TRAFFIC_SRC_SHA = "268812ecf5226308dae06647cd185d3da59b18180c4fceaf1e7d1989273d56b0"
 
 
 # the sources decode_kernel is compiled from
-DECODER_SOURCES = ["nlc_decode.cu", "nlc_decode_kernel.cuh", "nlc_tile.cuh", "nlc_tc.cuh",
-                   "nlc_model.cuh", "nlc_common.cuh", "nlc_kernels.cuh"]
+DECODER_SOURCES = ["nlc_decode.cu", "nlc_decode_kernel.cuh", "nlc_mma.cuh", "nlc_quad.cuh",
+                   "nlc_f32.cuh", "nlc_tile.cuh", "nlc_tc.cuh", "nlc_model.cuh", "nlc_common.cuh",
+                   "nlc_kernels.cuh"]
 
 
 def _csrc_sha():
@@ -756,7 +757,7 @@ def main():
     coding_us = {name: float(cnt[8 + i]) / npx0 / mhz
                  for i, name in enumerate(["setup", "cdf_search", "rans", "posterior"])}
     net_us = {name: float(cnt[13 + i]) / ctas / steps_T / mhz
-              for i, name in enumerate(["gather", "mma", "epilogue"])}
+              for i, name in enumerate(["gather", "hidden_layers", "head"])}
     phases = {"steps": steps_T, "ctas": ctas, "tiles_per_cta_step": float(cnt[5]) / ctas / steps_T,
               "network_us_per_step": net_us,
               "us_per_step_measured": 1000.0 * ms / steps_T,

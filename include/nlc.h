@@ -149,13 +149,15 @@ int nlc_sync_status(nlc_ctx* ctx, nlc_stream stream);
 int nlc_set_tuning(nlc_ctx* ctx, int px_per_cta, int max_ctas);
 
 /* Limits of the decoder's bounded waits (also the sampler's): polls of the
- * grid barrier between wavefront steps and of an MMA's completion before the
- * wait gives up (0 = the defaults, 2^25 and 2^22 polls, far beyond any
- * normal wait).  A wait that gives up records NLC_ERR_TIMEOUT in the
- * context's status and releases every CTA of the launch, which leaves the
- * decode loop (an MMA wait first waits, bounded, for the MMAs it issued);
- * the context stays usable.  Small limits exist to exercise that path: a
- * reduced MMA limit counts non-blocking tests of the completion. */
+ * grid barrier between wavefront steps and, in the BF16 network, of the
+ * exchange between two layers' MMAs before the wait gives up (0 = the
+ * defaults, 2^25 and 2^22 polls, far beyond any normal wait).  A wait that
+ * gives up records NLC_ERR_TIMEOUT in the context's status and releases every
+ * CTA of the launch, which leaves the decode loop (an exchange first waits,
+ * bounded, for the warps it shares the layer with); the context stays usable.
+ * Small limits exist to exercise that path: a reduced MMA limit counts
+ * non-blocking tests of the exchange, which without one is a hardware barrier
+ * of the warps involved. */
 int nlc_set_wait_limits(nlc_ctx* ctx, uint32_t grid_polls, uint32_t mma_polls);
 
 /* Decoder phase profile (per-step latency against the dependency-bound step
@@ -172,8 +174,7 @@ int nlc_set_wait_limits(nlc_ctx* ctx, uint32_t grid_polls, uint32_t mma_polls);
  *   within [3], for the pixels coded by warp 0: [8] mixture and channel
  *   set-up, [9] CDF symbol search, [10] rANS state update, [11] posterior
  *   update, [12] pixels; within [2], for thread 0 (BF16 network): [13]
- *   context gather, [14] tensor-core MMA issue to completion, [15] epilogues
- *   (TMEM loads, bias/ELU, operand stores, CTA barriers).
+ *   context gather, [14] the network's hidden layers, [15] its head.
  * Synchronises the device when reading or changing the mode. */
 int nlc_decode_profile(nlc_ctx* ctx, int enable, uint64_t* h_counters);
 

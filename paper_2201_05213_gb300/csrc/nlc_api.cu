@@ -551,10 +551,10 @@ extern "C" int nlc_decompress(nlc_ctx* x, const uint8_t* d_in, const uint64_t* d
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const DeviceModel m = model_view(x);
-  if (decode_smem_bytes(x->d, (int)b.units.size()) > 227 * 1024)
+  const bool ring = x->d.shear && schedule == NLC_SCHED_WAVEFRONT;
+  if (decode_smem_bytes(x->d, (int)b.units.size(), ring) > 227 * 1024)
     return fail(NLC_ERR_UNSUPPORTED, "too many coding units in one call (%zu)", b.units.size());
   CodecBufs cb;
-  const bool ring = x->d.shear && schedule == NLC_SCHED_WAVEFRONT;
   if (ring && b.ring_rows >= (1LL << 31) / kRingRowBytes)
     return fail(NLC_ERR_UNSUPPORTED, "batch too large for the sheared decoder's rings");
   size_t need = layout_bufs(b, nullptr, cb, x->d_status, false, ring);
@@ -603,10 +603,10 @@ extern "C" int nlc_sample(nlc_ctx* x, const nlc_image_out* outs, int n, int patc
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   const DeviceModel m = model_view(x);
-  if (decode_smem_bytes(x->d, (int)b.units.size()) > 227 * 1024)
+  const bool ring = x->d.shear && schedule == NLC_SCHED_WAVEFRONT;
+  if (decode_smem_bytes(x->d, (int)b.units.size(), ring) > 227 * 1024)
     return fail(NLC_ERR_UNSUPPORTED, "too many coding units in one call (%zu)", b.units.size());
   CodecBufs cb;
-  const bool ring = x->d.shear && schedule == NLC_SCHED_WAVEFRONT;
   if (ring && b.ring_rows >= (1LL << 31) / kRingRowBytes)
     return fail(NLC_ERR_UNSUPPORTED, "batch too large for the sheared decoder's rings");
   size_t need = layout_bufs(b, nullptr, cb, x->d_status, false, ring);
@@ -873,9 +873,9 @@ extern "C" int nlc_plan_decode(nlc_ctx* x, const nlc_image_out* outs, int n, int
   Batch b;
   rc = plan_batch(x->d, n, ptrs.data(), H.data(), W.data(), patch, layout, schedule, b);
   if (rc) return rc;
-  if (decode_smem_bytes(x->d, (int)b.units.size()) > 227 * 1024)
-    return fail(NLC_ERR_UNSUPPORTED, "too many coding units in one call (%zu)", b.units.size());
   const bool ring = x->d.shear && schedule == NLC_SCHED_WAVEFRONT;
+  if (decode_smem_bytes(x->d, (int)b.units.size(), ring) > 227 * 1024)
+    return fail(NLC_ERR_UNSUPPORTED, "too many coding units in one call (%zu)", b.units.size());
   if (ring && b.ring_rows >= (1LL << 31) / kRingRowBytes)
     return fail(NLC_ERR_UNSUPPORTED, "batch too large for the sheared decoder's rings");
   nlc_plan* p = new nlc_plan();

@@ -11,8 +11,16 @@ static int decode_threads_of(int prec) {
   return prec == PREC_BF16 ? decode_threads<PREC_BF16>() : decode_threads<PREC_FP32>();
 }
 
-size_t decode_smem_bytes(const Dims& d, int n_units) {
-  return tile_smem_bytes(d, n_units, decode_threads_of(d.prec) / kGW, true);
+// Pixels per tile: 64 for the FP32 network, 128 for the BF16 network (64 where a very large number of
+// units leaves no room for 128; a share beyond one tile takes several).
+static int decode_rows(const Dims& d, int n_units, bool win) {
+  if (d.prec != PREC_BF16) return kF32Rows;
+  return dec_carve(d, nullptr, n_units, kTileMax, win, nullptr) <= 227 * 1024 ? kTileMax
+                                                                              : kTileMax / 2;
+}
+
+size_t decode_smem_bytes(const Dims& d, int n_units, bool win) {
+  return dec_carve(d, nullptr, n_units, decode_rows(d, n_units, win), win, nullptr);
 }
 
 // The kernel for a launch; prof selects the instrumented build (decoding
@@ -30,7 +38,7 @@ static const void* decode_fn(int prec, bool sample = false, bool win = false, bo
 }
 
 int decode_max_grid(const DeviceModel& m, int n_units, int sm_count, bool sample, bool win) {
-  const size_t smem = decode_smem_bytes(m.d, n_units);
+  const size_t smem = decode_smem_bytes(m.d, n_units, win);
   // both builds (plain and instrumented) get the attribute, so that a plan
   // set up before profiling was switched on can launch either; the grid is
   // the smaller of their co-resident counts
@@ -76,10 +84,11 @@ cudaError_t launch_decode(const DeviceModel& m, const CodecBufs& b, const uint8_
   a.times = b.times;
   a.n_times = b.n_times;
   a.ring = b.ring;
+  a.rows = decode_rows(m.d, b.n_units, b.ring != nullptr && sched == SCHED_WAVEFRONT);
   a.spin_limit = b.spin_limit ? b.spin_limit : kSpinLimit;
   a.mma_limit = b.mma_limit ? b.mma_limit : kMbarSpin;
   const bool win = b.ring != nullptr && sched == SCHED_WAVEFRONT;
-  const size_t smem = decode_smem_bytes(m.d, b.n_units);
+  const size_t smem = decode_smem_bytes(m.d, b.n_units, win);
   const void* fn = decode_fn(m.d.prec, false, win, b.prof != nullptr);
   const int nt = decode_threads_of(m.d.prec);
   if (set_attr &&
@@ -113,10 +122,11 @@ cudaError_t launch_sample(const DeviceModel& m, const CodecBufs& b, int sched, i
   a.n_times = 0;
   a.seed = seed;
   a.ring = b.ring;
+  a.rows = decode_rows(m.d, b.n_units, b.ring != nullptr && sched == SCHED_WAVEFRONT);
   a.spin_limit = b.spin_limit ? b.spin_limit : kSpinLimit;
   a.mma_limit = b.mma_limit ? b.mma_limit : kMbarSpin;
   const bool win = b.ring != nullptr && sched == SCHED_WAVEFRONT;
-  const size_t smem = decode_smem_bytes(m.d, b.n_units);
+  const size_t smem = decode_smem_bytes(m.d, b.n_units, win);
   const void* fn = decode_fn(m.d.prec, true, win);
   const int nt = decode_threads_of(m.d.prec);
   if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=

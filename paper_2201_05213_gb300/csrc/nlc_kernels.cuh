@@ -104,7 +104,7 @@ int decode_max_grid(const DeviceModel& m, int n_units, int sm_count, bool sample
 // instead of streams: draws the batch's pixels from the model.
 cudaError_t launch_sample(const DeviceModel& m, const CodecBufs& b, int sched, int T, int grid,
                           unsigned long long seed, cudaStream_t s);
-size_t decode_smem_bytes(const Dims& d, int n_units);
+size_t decode_smem_bytes(const Dims& d, int n_units, bool win);
 cudaError_t launch_forward(const DeviceModel& m, const CodecBufs& b, float* params, float* bits,
                            int sm_count, cudaStream_t s);
 cudaError_t launch_tables(const DeviceModel& m, const float* params, const uint8_t* pixels,

@@ -57,6 +57,12 @@ __device__ void gather_f32(const Unit* units, const PixSlot* slots, int h, float
   }
 }
 
+// A compile-time integer as a value.
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
 __device__ __forceinline__ float elu_f(float x) { return x > 0.f ? x : expm1f(x); }
 
 // ---------------------------------------------------------------------

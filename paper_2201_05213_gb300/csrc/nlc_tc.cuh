@@ -2,13 +2,13 @@
 //
 // A tile is M = 128 pixels.  Each layer is one chain of
 // tcgen05.mma.cta_group::1.kind::f16 instructions (K = 16 per instruction,
-// FP32 accumulation in TMEM columns [0, 128)) issued by one thread; the
+// FP32 accumulation in TMEM columns [0, 160)) issued by one thread; the
 // accumulator is read back with tcgen05.ld by all warps (warp w reads TMEM
 // lanes 32(w%4)..+31, i.e. its rows, and 8-column chunks w/4, w/4 + NP, ...),
 // bias/ELU/residual are applied in registers, and the next layer's A
 // operand stays in tensor memory: each thread writes its row's BF16 pairs
-// with tcgen05.st into columns [128, 128 + C/2) (lane m = row m, column
-// 128 + k/2 = elements k, k+1), which the next tcgen05.mma reads as its A
+// with tcgen05.st into columns [160, 160 + C/2) (lane m = row m, column
+// 160 + k/2 = elements k, k+1), which the next tcgen05.mma reads as its A
 // operand (8 columns per K step).  The first layer's A operand (the context
 // tile) and every B operand (the weights) are in shared memory, in the
 // canonical no-swizzle K-major layout:
@@ -32,8 +32,8 @@ namespace nlc {
 
 constexpr int kTcM = 128;
 constexpr int kTileMax = 128;
-constexpr int kTmemCols = 256;  // accumulator [0, 128), A operand [128, 128 + C/2)
-constexpr int kAcol = 128;       // first TMEM column of the A operand
+constexpr int kTmemCols = 256;  // accumulator [0, 160), A operand [160, 160 + C/2)
+constexpr int kAcol = 160;       // first TMEM column of the A operand (the head has N <= 160)
 constexpr unsigned kMbarSpin = 1u << 22;
 
 __host__ __device__ inline int align_up(int x, int a) { return (x + a - 1) / a * a; }
