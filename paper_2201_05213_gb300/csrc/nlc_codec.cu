@@ -1,6 +1,7 @@
 // Codec kernels of the nlc library (sm_103a) other than the tile pipeline:
 // weight packing, the per-stream rANS encoder, container pack/parse and the
 // stage-level entry points used by the parity tests.
+#include "nlc_tc.cuh"
 #include "nlc_tile.cuh"
 
 namespace nlc {

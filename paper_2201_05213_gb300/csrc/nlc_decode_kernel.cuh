@@ -431,13 +431,13 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
         const long long c0 = PROF && tick.pc ? clock64() : 0;
         if constexpr (SHEAR)
           net_gather_win(a.units, t.wrow, a.ring, d, t.net, step, t.flag[3]);
-        else if (d.shear) net_gather_shear(t.slots, d, t.net, n);
-        else net_gather(t.slots, d, t.net, n);
+        else if (d.shear) net_gather<true>(t.slots, d, t.net, n);
+        else net_gather<false>(t.slots, d, t.net, n);
         __syncthreads();
         if (PROF && tick.pc) tick.pc[13] += clock64() - c0;
         net_ok = net_run<PROF>(d, t.net, SHEAR ? t.flag[2] : n, SHEAR, pc);
       } else {
-        f32_gather(t.slots, n, d, t.f32);
+        f32_gather<true>(t.slots, n, d, t.f32);
         __syncthreads();
         f32_run(d, t.f32, n);
       }

@@ -167,9 +167,9 @@ __device__ __forceinline__ void f32_run(const Dims& d, float* sm, int n) {
   else f32_layers<4, 4>(d, sm, n, 16);
 }
 
-// Context tile of the decoder's slots (Slot: px, i, j, Wu, row_bytes as in
-// DecSlot), feature-major.
-template <class Slot>
+// Context tile of the slots (Slot: px, i, j, Wu, row_bytes as in DecSlot),
+// feature-major.  kCoherent: the image is being decoded (loads through L2).
+template <bool kCoherent, class Slot>
 __device__ __forceinline__ void f32_gather(const Slot* slots, int n, const Dims& d, float* sm) {
   float* X = sm + f32_plan(d).u;
   const int h = d.h, ldm = f32_ldm(n), ntap = 2 * h * (h + 1), np = ldm - 4;
@@ -183,7 +183,8 @@ __device__ __forceinline__ void f32_gather(const Slot* slots, int n, const Dims&
       tap_offset(p, h, dy, dx);
       if (s.i + dy >= 0 && s.j + dx >= 0 && s.j + dx < s.Wu) {
         const uint8_t* px = s.px + (long long)dy * s.row_bytes + 3 * dx;
-        const int a = ld_cg_u8(px), b = ld_cg_u8(px + 1), c = ld_cg_u8(px + 2);
+        const int a = kCoherent ? ld_cg_u8(px) : px[0], b = kCoherent ? ld_cg_u8(px + 1) : px[1],
+                  c = kCoherent ? ld_cg_u8(px + 2) : px[2];
         v0 = __fdiv_rn((float)(2 * a - 255), 255.f);
         v1 = __fdiv_rn((float)(2 * b - 255), 255.f);
         v2 = __fdiv_rn((float)(2 * c - 255), 255.f);

@@ -23,6 +23,7 @@
 // among its m-tile's warps.  The residual stream stays in FP32 registers.
 #pragma once
 
+#include "nlc_model.cuh"
 #include "nlc_tc.cuh"
 
 namespace nlc {
@@ -408,96 +409,104 @@ __device__ __forceinline__ float byte_input(uint32_t w, int k) {
   return __fmaf_rn(__fsub_rn(f, kFixOne), 2.f, -255.f);
 }
 
-// Masked tile: X(m, k) = 2v - 255 for feature k = 3p + c of tap p, 0 outside
-// the unit and for F <= k < Fp.  One lane per (pixel m, context row r): row r
-// < h is image row i - h + r over columns j-h .. j+h, row h is row i over
-// columns j-h .. j-1; its bytes are contiguous in the image and are read as
-// the aligned 32-bit words that hold at least one byte of the row inside the
-// unit, realigned with funnel shifts.  A warp covers 8 pixels x 4 rows.
-static __device__ __noinline__ void net_gather(const DecSlot* slots, const Dims& d, NetSmem& t,
-                                               int n) {
-  const int h = d.h, Fp = d.Fp, F = d.F, w2 = 2 * h + 1, rows = t.rows;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = lane >> 3;
-  for (int mb = 8 * warp; mb < n; mb += 8 * (int)(blockDim.x >> 5)) {
-    const int m = mb + (lane & 7);
-    if (r > h || m >= n) continue;
-    const DecSlot s = slots[m];
-    const int ncol = r < h ? w2 : h;  // pixels of this row's window
-    const int k0 = 3 * r * w2;
-    // window columns x = j - h + c, c in [0, ncol); inside the unit: [ca, cb)
-    const int x0 = s.j - h;
-    const int ca = x0 < 0 ? -x0 : 0;
-    const int cb = min(ncol, s.Wu - x0);
-    const bool row_ok = s.i - h + r >= 0 && ca < cb;
-    uint32_t wv[7] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    uint32_t sh = 0;
-    if (row_ok) {
-      const uintptr_t lo = (uintptr_t)(s.px + (long long)(r - h) * s.row_bytes - 3 * h);
-      const uintptr_t a = lo + 3 * ca, b = lo + 3 * cb;  // bytes inside the unit
-      const uintptr_t w0 = lo & ~(uintptr_t)3;
-      sh = 8u * (uint32_t)(lo & 3);
-#pragma unroll
-      for (int q = 0; q < 6; q++) {
-        const uintptr_t wa = w0 + 4 * q;
-        if (wa + 4 > a && wa < b) wv[q] = ld_cg_u32(reinterpret_cast<const uint32_t*>(wa));
-      }
-    }
-    uint32_t al[6];
-#pragma unroll
-    for (int q = 0; q < 6; q++) al[q] = __funnelshift_r(wv[q], wv[q + 1], sh);
-    uint16_t* X = t.X + 8 * m;
-#pragma unroll
-    for (int q = 0; q < 3 * (2 * kMaxH + 1); q++) {
-      const int c = q / 3;
-      if (c < ncol) {
-        const float x = (row_ok && c >= ca && c < cb) ? byte_input(al[q >> 2], q & 3) : 0.f;
-        const int k = k0 + q;
-        X[(k >> 3) * 8 * rows + (k & 7)] = __bfloat16_as_ushort(__float2bfloat16_rn(x));
-      }
-    }
-    if (r == h)
-      for (int k = F; k < Fp; k++) X[(k >> 3) * 8 * rows + (k & 7)] = 0;
-  }
+template <bool kCoherent>
+__device__ __forceinline__ uint32_t ld_px_word(uintptr_t a) {
+  const uint32_t* p = reinterpret_cast<const uint32_t*>(a);
+  return kCoherent ? ld_cg_u32(p) : __ldg(p);
 }
 
-// Sheared model, per-pixel window rows (raster and sequential decoding):
-// window row dd's features in chunks dd * Fsp/8 onwards.
-static __device__ __noinline__ void net_gather_shear(const DecSlot* slots, const Dims& d,
-                                                     NetSmem& t, int n) {
-  const int h = d.h, Ws = d.Ws, Fsp = d.Fsp, rows = t.rows;
+// Masked tile: X(m, k) = 2v - 255 for feature k = 3p + c of tap p, 0 outside
+// the unit and for F <= k < Fp.  One lane per (pixel, context row r): row r <
+// h is image row i - h + r over columns j-h .. j+h, row h is row i over
+// columns j-h .. j-1; its bytes are contiguous in the image and are read as
+// the aligned 32-bit words that hold at least one byte of the row inside the
+// unit, realigned with funnel shifts.  X: the pixel's row of the first chunk,
+// cs: elements from one chunk to the next.
+template <bool kCoherent, class Slot>
+__device__ __forceinline__ void gather_row(const Slot& s, int r, int h, int F, int Fp, uint16_t* X,
+                                           int cs) {
+  const int w2 = 2 * h + 1;
+  const int ncol = r < h ? w2 : h;  // pixels of this row's window
+  const int k0 = 3 * r * w2;
+  // window columns x = j - h + c, c in [0, ncol); inside the unit: [ca, cb)
+  const int x0 = s.j - h;
+  const int ca = x0 < 0 ? -x0 : 0;
+  const int cb = min(ncol, s.Wu - x0);
+  const bool row_ok = s.i - h + r >= 0 && ca < cb;
+  uint32_t wv[7] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  uint32_t sh = 0;
+  if (row_ok) {
+    const uintptr_t lo = (uintptr_t)(s.px + (long long)(r - h) * s.row_bytes - 3 * h);
+    const uintptr_t a = lo + 3 * ca, b = lo + 3 * cb;  // bytes inside the unit
+    const uintptr_t w0 = lo & ~(uintptr_t)3;
+    sh = 8u * (uint32_t)(lo & 3);
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      const uintptr_t wa = w0 + 4 * q;
+      if (wa + 4 > a && wa < b) wv[q] = ld_px_word<kCoherent>(wa);
+    }
+  }
+  uint32_t al[6];
+#pragma unroll
+  for (int q = 0; q < 6; q++) al[q] = __funnelshift_r(wv[q], wv[q + 1], sh);
+#pragma unroll
+  for (int q = 0; q < 3 * (2 * kMaxH + 1); q++) {
+    const int c = q / 3;
+    if (c < ncol) {
+      const float x = (row_ok && c >= ca && c < cb) ? byte_input(al[q >> 2], q & 3) : 0.f;
+      const int k = k0 + q;
+      X[(k >> 3) * cs + (k & 7)] = __bfloat16_as_ushort(__float2bfloat16_rn(x));
+    }
+  }
+  if (r == h)
+    for (int k = F; k < Fp; k++) X[(k >> 3) * cs + (k & 7)] = 0;
+}
+
+// Sheared model, per-pixel window row dd: its Fsp features from chunk
+// dd * Fsp/8 onwards (X: the pixel's row of that chunk).
+template <bool kCoherent, class Slot>
+__device__ __forceinline__ void gather_row_shear(const Slot& s, int dd, int h, int Ws, int Fsp,
+                                                 uint16_t* X, int cs) {
+  const int dx = (h + 1) * (h - dd) - Ws;  // window column 0 from the pixel's column
+  const int x0 = s.j + dx;
+  const int ca = x0 < 0 ? -x0 : 0;
+  const int cb = min(Ws, s.Wu - x0);
+  const bool row_ok = s.i - h + dd >= 0 && ca < cb;
+  uint32_t wv[13];
+#pragma unroll
+  for (int q = 0; q < 13; q++) wv[q] = 0u;
+  uint32_t sh = 0;
+  if (row_ok) {
+    const uintptr_t lo = (uintptr_t)(s.px + (long long)(dd - h) * s.row_bytes + 3 * dx);
+    const uintptr_t a = lo + 3 * ca, b = lo + 3 * cb;
+    const uintptr_t w0 = lo & ~(uintptr_t)3;
+    sh = 8u * (uint32_t)(lo & 3);
+#pragma unroll
+    for (int q = 0; q < 13; q++) {
+      const uintptr_t wa = w0 + 4 * q;
+      if (wa + 4 > a && wa < b) wv[q] = ld_px_word<kCoherent>(wa);
+    }
+  }
+  uint32_t al[12];
+#pragma unroll
+  for (int q = 0; q < 12; q++) al[q] = __funnelshift_r(wv[q], wv[q + 1], sh);
+  shear_row_features(al, Ws, Fsp, ca, cb, row_ok,
+                     [&](int kc) { return reinterpret_cast<uint4*>(X + kc * cs); });
+}
+
+// The decoder's tile, from its slots: a warp covers 8 pixels x 4 rows.
+template <bool SHEAR>
+__device__ __noinline__ void net_gather(const DecSlot* slots, const Dims& d, NetSmem& t, int n) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int dd = lane >> 3;
+  const int r = lane >> 3, cs = 8 * t.rows;
   for (int mb = 8 * warp; mb < n; mb += 8 * (int)(blockDim.x >> 5)) {
     const int m = mb + (lane & 7);
-    if (dd > h || m >= n) continue;
+    if (r > d.h || m >= n) continue;
     const DecSlot s = slots[m];
-    const int dx = (h + 1) * (h - dd) - Ws;  // window column 0 from the pixel's column
-    const int x0 = s.j + dx;
-    const int ca = x0 < 0 ? -x0 : 0;
-    const int cb = min(Ws, s.Wu - x0);
-    const bool row_ok = s.i - h + dd >= 0 && ca < cb;
-    uint32_t wv[13];
-#pragma unroll
-    for (int q = 0; q < 13; q++) wv[q] = 0u;
-    uint32_t sh = 0;
-    if (row_ok) {
-      const uintptr_t lo = (uintptr_t)(s.px + (long long)(dd - h) * s.row_bytes + 3 * dx);
-      const uintptr_t a = lo + 3 * ca, b = lo + 3 * cb;
-      const uintptr_t w0 = lo & ~(uintptr_t)3;
-      sh = 8u * (uint32_t)(lo & 3);
-#pragma unroll
-      for (int q = 0; q < 13; q++) {
-        const uintptr_t wa = w0 + 4 * q;
-        if (wa + 4 > a && wa < b) wv[q] = ld_cg_u32(reinterpret_cast<const uint32_t*>(wa));
-      }
-    }
-    uint32_t al[12];
-#pragma unroll
-    for (int q = 0; q < 12; q++) al[q] = __funnelshift_r(wv[q], wv[q + 1], sh);
-    uint16_t* X = t.X + (size_t)dd * (Fsp / 8) * 8 * rows + 8 * m;
-    shear_row_features(al, Ws, Fsp, ca, cb, row_ok,
-                       [&](int kc) { return reinterpret_cast<uint4*>(X + kc * 8 * rows); });
+    if (SHEAR)
+      gather_row_shear<true>(s, r, d.h, d.Ws, d.Fsp, t.X + (size_t)r * (d.Fsp / 8) * cs + 8 * m, cs);
+    else
+      gather_row<true>(s, r, d.h, d.F, d.Fp, t.X + 8 * m, cs);
   }
 }
 

@@ -183,4 +183,41 @@ __device__ __forceinline__ void quad_pair(const QuadChan<KI>& o, int v, uint32_t
   c1 = cum_fix(F1, v + 1);
 }
 
+// Model code length: adds log P(v[CH]) of channel CH to the components'
+// running log-likelihoods l (the locations are not bounded here).
+template <int CH, int KI, class Param>
+__device__ __forceinline__ void quad_loglik(Param P, int K, int q, const int (&v)[3],
+                                            float (&l)[KI]) {
+  const float xr = xval_f(v[0]), xg = xval_f(v[1]);
+#pragma unroll
+  for (int i = 0; i < KI; i++) {
+    if (q + 4 * i >= K) continue;
+    float m = P(1 + CH, i);
+    if (CH == 1) m = __fadd_rn(m, __fmul_rn(tanh_f(P(7, i)), xr));
+    if (CH == 2)
+      m = __fadd_rn(__fadd_rn(m, __fmul_rn(tanh_f(P(8, i)), xr)), __fmul_rn(tanh_f(P(9, i)), xg));
+    const float ls = fmaxf(P(4 + CH, i), -7.f), inv = exp_f(-ls);
+    l[i] = __fadd_rn(l[i], log_bin_mass_f(m, inv, bin_log_width(ls, inv), v[CH]));
+  }
+}
+
+// -log2 sum_k e^{l_k}; the sum pairs components 8, then 4, 2, 1 apart (the
+// butterfly of a 16-lane group with one component per lane).
+template <int KI>
+__device__ __forceinline__ float quad_bits(const float (&l)[KI], int K, int q) {
+  float mx = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < KI; i++)
+    if (q + 4 * i < K) mx = fmaxf(mx, l[i]);
+  mx = quad_max(mx);
+  float e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < KI; i++)
+    if (q + 4 * i < K) e[i] = expf(__fsub_rn(l[i], mx));
+  float s = __fadd_rn(__fadd_rn(e[0], e[2]), __fadd_rn(e[1], e[3]));
+  s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 2));
+  s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 1));
+  return -__fadd_rn(mx, logf(s)) * 1.4426950408889634f;
+}
+
 }  // namespace nlc

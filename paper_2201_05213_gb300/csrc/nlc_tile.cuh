@@ -1,6 +1,5 @@
 // Device helpers shared by the codec kernels: unit lookup, block scans, the
-// warp-level rANS decoder, the per-stream rANS encoder and the tile pipeline
-// (gather -> local network) in shared memory.
+// rANS decoder of a coding group and the per-stream rANS encoder.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -9,11 +8,8 @@
 #include "nlc_common.cuh"
 #include "nlc_kernels.cuh"
 #include "nlc_model.cuh"
-#include "nlc_tc.cuh"
 
 namespace nlc {
-
-constexpr int kMT = 64;  // pixels per tile of the FP32 pipeline
 
 // ---------------------------------------------------------------------
 // Shared helpers
@@ -104,7 +100,7 @@ __device__ __forceinline__ int front_scan(const Unit* __restrict__ units, int n_
 // rANS: warp-level decoder of one stream position and the per-stream
 // encoder (byte-wise renormalisation, state in [2^23, 2^31)).
 // ---------------------------------------------------------------------
-// Coding groups of the codec kernels: 16 lanes (half a warp) per pixel.
+// Coding groups of the table entry point: 16 lanes (half a warp) per pixel.
 constexpr int kGW = 16;
 constexpr int kGroups = kThreads / kGW;
 
@@ -202,140 +198,6 @@ __device__ __forceinline__ int rans_encode_stream(Get get, long long nsym, uint8
   *--w = (uint8_t)(x >> 24);
   return (int)(slot_end - w);
 }
-
-// ---------------------------------------------------------------------
-// Tile pipeline (FP32 SIMT network) shared by encode, decode and forward.
-// ---------------------------------------------------------------------
-struct TileSmem {
-  float* Wt;
-  float* A;
-  float* B1;
-  float* U0;
-  WarpScratch* ws;
-  PixSlot* slots;
-  int* pre;
-  StreamRec* rec;  // decoder: the tile's stream records (kTileMax)
-  uint32_t* win;   // decoder: per pixel, the 12 stream bytes from pos + 8, word-aligned
-  int* prow;       // sheared wavefront decoder: output row of the tile's pixel s
-  int* rofs;       // sheared wavefront decoder: ring byte offset of the tile's pixel s
-  int2* wrow;      // sheared wavefront decoder: (unit, unit row) of window row rho
-  long long* sh;
-  long long* pc;  // 16 profiling accumulators (thread 0 only)
-  int* flag;
-  TcSmem tc;
-};
-
-// Network outputs of the tile's m-th pixel.
-__device__ __forceinline__ const float* tile_params(const TileSmem& t, const Dims& d, int m) {
-  return t.U0 + (size_t)m * d.ldP;
-}
-
-// Shared memory of the tile pipeline with `groups` coding groups (and, for
-// the decoder, the tile's stream records and windows).
-__host__ __device__ inline size_t tile_smem_bytes(const Dims& d, int n_pre, int groups = kGroups,
-                                                  bool dec = false) {
-  size_t bytes;
-  if (d.prec == PREC_BF16) {
-    bytes = tc_smem_bytes(d);
-  } else {
-    SimtPlan pl = simt_plan(d, (int)simt_floats(d), kMT);
-    bytes = (size_t)pl.end * 4;
-  }
-  bytes = (bytes + 15) & ~(size_t)15;
-  bytes += sizeof(WarpScratch) * groups;
-  if (dec) bytes += (sizeof(StreamRec) + 4 * sizeof(uint32_t) + 2 * sizeof(int)) * kTileMax +
-                    sizeof(int2) * kWinRows;
-  bytes += sizeof(PixSlot) * kTileMax;
-  bytes += sizeof(long long) * (33 + 16);
-  bytes += sizeof(int) * (n_pre + 1 + 4);
-  return (bytes + 15) & ~(size_t)15;
-}
-
-__device__ __forceinline__ TileSmem carve(const Dims& d, unsigned char* smem, int n_pre,
-                                          int groups = kGroups, bool dec = false) {
-  TileSmem t;
-  size_t off;
-  if (d.prec == PREC_BF16) {
-    t.tc = tc_carve(d, smem);
-    off = tc_smem_bytes(d);
-    t.Wt = t.A = t.B1 = nullptr;
-    t.U0 = t.tc.P;
-  } else {
-    SimtPlan pl = simt_plan(d, (int)simt_floats(d), kMT);
-    float* f = reinterpret_cast<float*>(smem);
-    t.Wt = f + pl.w_off;
-    t.A = f + pl.a_off;
-    t.B1 = f + pl.b1_off;
-    t.U0 = f + pl.u0_off;
-    off = (size_t)pl.end * 4;
-  }
-  off = (off + 15) & ~(size_t)15;
-  t.ws = reinterpret_cast<WarpScratch*>(smem + off);
-  off += sizeof(WarpScratch) * groups;
-  t.rec = nullptr;
-  t.win = nullptr;
-  t.prow = nullptr;
-  t.rofs = nullptr;
-  t.wrow = nullptr;
-  if (dec) {
-    t.rec = reinterpret_cast<StreamRec*>(smem + off);
-    off += sizeof(StreamRec) * kTileMax;
-    t.win = reinterpret_cast<uint32_t*>(smem + off);
-    off += 4 * sizeof(uint32_t) * kTileMax;
-    t.wrow = reinterpret_cast<int2*>(smem + off);
-    off += sizeof(int2) * kWinRows;
-    t.prow = reinterpret_cast<int*>(smem + off);
-    off += sizeof(int) * kTileMax;
-    t.rofs = reinterpret_cast<int*>(smem + off);
-    off += sizeof(int) * kTileMax;
-  }
-  t.slots = reinterpret_cast<PixSlot*>(smem + off);
-  off += sizeof(PixSlot) * kTileMax;
-  t.sh = reinterpret_cast<long long*>(smem + off);
-  off += sizeof(long long) * 33;
-  t.pc = reinterpret_cast<long long*>(smem + off);
-  off += sizeof(long long) * 16;
-  t.pre = reinterpret_cast<int*>(smem + off);
-  t.flag = t.pre + n_pre + 1;
-  (void)n_pre;
-  return t;
-}
-
-template <int PREC>
-__device__ __forceinline__ constexpr int tile_size() { return PREC == PREC_BF16 ? kTcM : kMT; }
-
-template <int PREC>
-__device__ __forceinline__ void load_weights(const DeviceModel& m, TileSmem& t) {
-  if constexpr (PREC == PREC_BF16) {
-    tc_load_weights(m.d, m.w, t.tc);
-  } else {
-    const int n = m.w.simt_floats;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) t.Wt[i] = m.w.simt[i];
-  }
-}
-
-// gather + network for the slots of the tile; P[m][NOp] lands in t.U0.
-// With pc non-null (BF16), thread 0 adds its gather cycles to pc[13] and the
-// network's sub-phases to pc[14], pc[15] (shared-memory accumulators).
-// Returns false (in every thread) if an MMA completion wait timed out.
-template <int PREC, bool kCoherent, int NT = kThreads>
-__device__ __forceinline__ bool tile_network(const DeviceModel& m, const Unit* units, TileSmem& t,
-                                             int n_valid, long long* pc = nullptr) {
-  if constexpr (PREC == PREC_BF16) {
-    const long long c0 = pc != nullptr && threadIdx.x == 0 ? clock64() : 0;
-    if (m.d.shear) tc_gather_shear_px<kCoherent>(units, t.slots, m.d, t.tc, n_valid);
-    else tc_gather<kCoherent>(units, t.slots, m.d, t.tc, n_valid);
-    __syncthreads();
-    if (pc != nullptr && threadIdx.x == 0) pc[13] += clock64() - c0;
-    return tc_network<NT>(m.d, t.tc, n_valid, pc);
-  } else {
-    gather_f32<kMT, kCoherent>(units, t.slots, m.d.h, t.U0);
-    __syncthreads();
-    network_simt_run<kMT>(m.d, t.Wt, t.A, t.B1, t.U0);
-    return true;
-  }
-}
-
 
 __device__ __forceinline__ int unit_streams(const Unit& U, int layout) {
   return layout == 1 ? U.Hu : 1;
