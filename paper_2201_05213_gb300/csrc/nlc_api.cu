@@ -710,8 +710,8 @@ static int run_adjoint(nlc_ctx* x, const uint8_t* d_batch, int N, int H, int W,
     CUDA_TRY(launch_tc_train(x->d, x->d_umma, x->d_bias, d_batch, N, H, W, d_dparams, d_loss,
                              d_grad, x->ws, x->sm_count, x->d_status, s));
   else
-    CUDA_TRY(launch_loss_grad(x->d, x->d_w, x->d_simt, d_batch, N, H, W, d_dparams, d_loss,
-                              d_grad, x->ws, x->sm_count, s));
+    CUDA_TRY(launch_loss_grad(x->d, x->d_simt, d_batch, N, H, W, d_dparams, d_loss, d_grad, x->ws,
+                              x->sm_count, s));
   return NLC_OK;
 }
 

@@ -52,29 +52,34 @@ __device__ __forceinline__ void f32_load(const float* p, float (&v)[N]) {
     const float2 x = *reinterpret_cast<const float2*>(p);
     v[0] = x.x, v[1] = x.y;
   } else {
-    v[0] = *p;
+#pragma unroll
+    for (int i = 0; i < N; i++) v[i] = p[i];
   }
 }
 
-// acc[b][a] += w[k][b] in[k][a] for the U inputs k0 .. (all loads, then the FMAs).
+// The operands of U inputs, and their multiply-adds.
 template <int U, int PX, int NB>
-__device__ __forceinline__ void f32_step(const float* in, int ldm, const float* w, int N,
-                                         float (&acc)[NB][PX]) {
+struct F32Step {
   float x[U][PX], v[U][NB];
+  __device__ __forceinline__ void load(const float* in, int ldm, const float* w, int N) {
 #pragma unroll
-  for (int k = 0; k < U; k++) {
-    f32_load<PX>(in + k * ldm, x[k]);
-    f32_load<NB>(w + k * N, v[k]);
+    for (int k = 0; k < U; k++) {
+      f32_load<PX>(in + k * ldm, x[k]);
+      f32_load<NB>(w + k * N, v[k]);
+    }
   }
+  __device__ __forceinline__ void fma(float (&acc)[NB][PX]) const {
 #pragma unroll
-  for (int k = 0; k < U; k++)
+    for (int k = 0; k < U; k++)
 #pragma unroll
-    for (int b = 0; b < NB; b++)
+      for (int b = 0; b < NB; b++)
 #pragma unroll
-      for (int a = 0; a < PX; a++) acc[b][a] = __fmaf_rn(x[k][a], v[k][b], acc[b][a]);
-}
+        for (int a = 0; a < PX; a++) acc[b][a] = __fmaf_rn(x[k][a], v[k][b], acc[b][a]);
+  }
+};
 
 // acc[b][a] = sum over k < Kd (a multiple of 4), ascending, of w[k][b] in[k][a].
+// The next four inputs are read while the present ones are multiplied.
 template <int PX, int NB>
 __device__ __forceinline__ void f32_dot(const float* in, int ldm, int Kd, const float* w, int N,
                                         float (&acc)[NB][PX]) {
@@ -82,11 +87,23 @@ __device__ __forceinline__ void f32_dot(const float* in, int ldm, int Kd, const 
   for (int b = 0; b < NB; b++)
 #pragma unroll
     for (int a = 0; a < PX; a++) acc[b][a] = 0.f;
-  constexpr int U = PX * NB >= 16 ? 4 : 8;
-  int k = 0;
+  F32Step<4, PX, NB> s0, s1;
+  s0.load(in, ldm, w, N);
+  int k = 4;
 #pragma unroll 1
-  for (; k + U <= Kd; k += U) f32_step<U, PX, NB>(in + k * ldm, ldm, w + k * N, N, acc);
-  if (U > 4 && k < Kd) f32_step<4, PX, NB>(in + k * ldm, ldm, w + k * N, N, acc);
+  for (; k + 4 < Kd; k += 8) {
+    s1.load(in + k * ldm, ldm, w + k * N, N);
+    s0.fma(acc);
+    s0.load(in + (k + 4) * ldm, ldm, w + (k + 4) * N, N);
+    s1.fma(acc);
+  }
+  if (k < Kd) {
+    s1.load(in + k * ldm, ldm, w + k * N, N);
+    s0.fma(acc);
+    s1.fma(acc);
+  } else {
+    s0.fma(acc);
+  }
 }
 
 // X (features of n pixels, stride f32_ldm(n)) -> P[m][ldP]; the caller's

@@ -10,13 +10,6 @@
 
 namespace nlc {
 
-// One pixel slot of a tile.
-struct PixSlot {
-  int unit;   // unit index, -1 for an empty slot
-  int i, j;   // position inside the unit
-  int aux;    // decoder: stream index; encoder: pixel index in the batch
-};
-
 // ---------------------------------------------------------------------
 // Context gather (Eq. 3): taps p enumerate rows dy=-h..-1 with dx=-h..h,
 // then dy=0 with dx=-h..-1; feature 3p+c holds channel c.  Outside the
@@ -28,35 +21,6 @@ __device__ __forceinline__ void tap_offset(int p, int h, int& dy, int& dx) {
   dx = p % w - h;
 }
 
-// FP32 layout: X[f][m] (feature-major), value (2v-255)/255.
-template <int MT, bool kCoherent>
-__device__ void gather_f32(const Unit* units, const PixSlot* slots, int h, float* X) {
-  const int ntap = 2 * h * (h + 1);
-  for (int it = threadIdx.x; it < MT * ntap; it += blockDim.x) {
-    int m = it % MT, p = it / MT;
-    const PixSlot s = slots[m];
-    float v0 = 0.f, v1 = 0.f, v2 = 0.f;
-    if (s.unit >= 0) {
-      const Unit u = units[s.unit];
-      int dy, dx;
-      tap_offset(p, h, dy, dx);
-      int ii = s.i + dy, jj = s.j + dx;
-      if (ii >= 0 && ii < u.Hu && jj >= 0 && jj < u.Wu) {
-        const uint8_t* px = u.img + ((long long)(u.y0 + ii) * u.img_W + (u.x0 + jj)) * 3;
-        int a, b, c;
-        if (kCoherent) { a = ld_cg_u8(px); b = ld_cg_u8(px + 1); c = ld_cg_u8(px + 2); }
-        else { a = px[0]; b = px[1]; c = px[2]; }
-        v0 = __fdiv_rn((float)(2 * a - 255), 255.f);
-        v1 = __fdiv_rn((float)(2 * b - 255), 255.f);
-        v2 = __fdiv_rn((float)(2 * c - 255), 255.f);
-      }
-    }
-    X[(3 * p + 0) * MT + m] = v0;
-    X[(3 * p + 1) * MT + m] = v1;
-    X[(3 * p + 2) * MT + m] = v2;
-  }
-}
-
 // A compile-time integer as a value.
 template <int V>
 struct IntC {
@@ -65,139 +29,11 @@ struct IntC {
 
 __device__ __forceinline__ float elu_f(float x) { return x > 0.f ? x : expm1f(x); }
 
-// ---------------------------------------------------------------------
-// FP32 SIMT local network.  Activations are feature-major [n][m]; each
-// thread owns 4 pixels x NB outputs (N = 16 NB), accumulating over k in
-// ascending order with explicit fma.
-// ---------------------------------------------------------------------
-enum GemmMode { GM_STORE = 0, GM_ELU = 1, GM_RESID = 2, GM_HEAD = 3 };
-
-template <int MT, int NB, int MODE>
-__device__ __noinline__ void gemm_simt(const float* __restrict__ in, int Kd,
-                                          const float* __restrict__ WT,
-                                          const float* __restrict__ bias, float* __restrict__ out,
-                                          int ldp) {
-  static_assert(MT == 64, "the SIMT tile is 64 pixels");
-  constexpr int N = 16 * NB;
-  const int tm = threadIdx.x & 15, tn = threadIdx.x >> 4;
-  const int m0 = tm * 4, n0 = tn * NB;
-  float acc[4][NB];
-#pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int b = 0; b < NB; b++) acc[a][b] = 0.f;
-  for (int k = 0; k < Kd; k++) {
-    const float4 x = *reinterpret_cast<const float4*>(in + k * MT + m0);
-    const float* wr = WT + k * N + n0;
-    float wv[NB];
-#pragma unroll
-    for (int b = 0; b < NB; b++) wv[b] = wr[b];
-#pragma unroll
-    for (int b = 0; b < NB; b++) {
-      acc[0][b] = __fmaf_rn(x.x, wv[b], acc[0][b]);
-      acc[1][b] = __fmaf_rn(x.y, wv[b], acc[1][b]);
-      acc[2][b] = __fmaf_rn(x.z, wv[b], acc[2][b]);
-      acc[3][b] = __fmaf_rn(x.w, wv[b], acc[3][b]);
-    }
-  }
-#pragma unroll
-  for (int b = 0; b < NB; b++) {
-    const float bb = bias[n0 + b];
-#pragma unroll
-    for (int a = 0; a < 4; a++) {
-      float v = __fadd_rn(acc[a][b], bb);
-      if (MODE == GM_STORE) out[(n0 + b) * MT + m0 + a] = v;
-      if (MODE == GM_ELU) out[(n0 + b) * MT + m0 + a] = elu_f(v);
-      if (MODE == GM_RESID) {
-        float* o = out + (n0 + b) * MT + m0 + a;
-        *o = __fadd_rn(*o, v);
-      }
-      if (MODE == GM_HEAD) out[(m0 + a) * ldp + n0 + b] = v;
-    }
-  }
-}
-
-template <int MT, int NB>
-__device__ __forceinline__ void gemm_layer(int mode, const float* in, int Kd, const float* WT,
-                                           const float* bias, float* out, int ldp) {
-  switch (mode) {
-    case GM_STORE: gemm_simt<MT, NB, GM_STORE>(in, Kd, WT, bias, out, ldp); break;
-    case GM_ELU: gemm_simt<MT, NB, GM_ELU>(in, Kd, WT, bias, out, ldp); break;
-    case GM_RESID: gemm_simt<MT, NB, GM_RESID>(in, Kd, WT, bias, out, ldp); break;
-    default: gemm_simt<MT, NB, GM_HEAD>(in, Kd, WT, bias, out, ldp); break;
-  }
-}
-
-template <int MT>
-__device__ void gemm_dispatch(int mode, const float* in, int Kd, const float* WT, const float* bias,
-                              int N, float* out, int ldp) {
-  switch (N / 16) {
-    case 1: gemm_layer<MT, 1>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 2: gemm_layer<MT, 2>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 3: gemm_layer<MT, 3>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 4: gemm_layer<MT, 4>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 5: gemm_layer<MT, 5>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 6: gemm_layer<MT, 6>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 7: gemm_layer<MT, 7>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 8: gemm_layer<MT, 8>(mode, in, Kd, WT, bias, out, ldp); break;
-    case 9: gemm_layer<MT, 9>(mode, in, Kd, WT, bias, out, ldp); break;
-    default: gemm_layer<MT, 10>(mode, in, Kd, WT, bias, out, ldp); break;
-  }
-}
-
 // Floats of the packed FP32 weights:
 // W0T[F][C] b0[C] {W1T[C][C] b1[C] W2T[C][C] b2[C]} x R WHT[C][NOp] bH[NOp].
 __host__ __device__ inline size_t simt_floats(const Dims& d) {
   return (size_t)d.F * d.C + d.C + (size_t)d.R * (2 * d.C * d.C + 2 * d.C) + (size_t)d.C * d.NOp +
          d.NOp;
-}
-
-// Shared-memory plan of the FP32 tile pipeline (all offsets in floats).
-struct SimtPlan {
-  int w_off, a_off, b1_off, u0_off, end;
-};
-
-__host__ __device__ inline SimtPlan simt_plan(const Dims& d, int simt_floats, int MT) {
-  SimtPlan p;
-  int u0 = d.Fp * MT;
-  if (d.C * MT > u0) u0 = d.C * MT;
-  if (MT * d.ldP > u0) u0 = MT * d.ldP;
-  p.w_off = 0;
-  p.a_off = (simt_floats + 3) & ~3;
-  p.b1_off = p.a_off + d.C * MT;
-  p.u0_off = p.b1_off + d.C * MT;
-  p.end = p.u0_off + u0;
-  return p;
-}
-
-// Network of a 64-pixel tile: X (features, in U0) -> P[m][ldP] (in U0).
-template <int MT>
-__device__ void network_simt_run(const Dims& d, const float* Wt, float* A, float* B1, float* U0) {
-  const int C = d.C, F = d.F;
-  const float* W0T = Wt;
-  const float* b0 = W0T + F * C;
-  const float* cur = b0 + C;
-  gemm_dispatch<MT>(GM_STORE, U0, F, W0T, b0, C, A, 0);
-  __syncthreads();
-  for (int r = 0; r < d.R; r++) {
-    const float* W1T = cur;
-    const float* b1 = W1T + C * C;
-    const float* W2T = b1 + C;
-    const float* b2 = W2T + C * C;
-    cur = b2 + C;
-    for (int e = threadIdx.x; e < C * MT; e += blockDim.x) B1[e] = elu_f(A[e]);
-    __syncthreads();
-    gemm_dispatch<MT>(GM_ELU, B1, C, W1T, b1, C, U0, 0);
-    __syncthreads();
-    gemm_dispatch<MT>(GM_RESID, U0, C, W2T, b2, C, A, 0);
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < C * MT; e += blockDim.x) B1[e] = elu_f(A[e]);
-  __syncthreads();
-  const float* WHT = cur;
-  const float* bH = WHT + C * d.NOp;
-  gemm_dispatch<MT>(GM_HEAD, B1, C, WHT, bH, d.NOp, U0, d.ldP);
-  __syncthreads();
 }
 
 // ---------------------------------------------------------------------

@@ -1,5 +1,5 @@
 // Maximum-likelihood training of the local model (Eq. 2): one fused kernel
-// runs, per 64-pixel tile, the forward pass, the mixture NLL with its
+// runs, per 32-pixel tile, the forward pass, the mixture NLL with its
 // analytic gradient, and the adjoint of the 1x1 residual blocks and of the
 // masked first layer; weight gradients accumulate in a per-CTA slot that a
 // second kernel reduces in a fixed order (deterministic).
@@ -7,386 +7,632 @@
 #include <stdint.h>
 
 #include "nlc_common.cuh"
+#include "nlc_f32.cuh"
 #include "nlc_model.cuh"
 #include "nlc_train.cuh"
 
 namespace nlc {
 
-constexpr int kTM = 64;
+// A tile is 16 PX pixels (PX = 2, or 1 for models whose weights leave no room
+// for more); its feature-major tiles have rows of 16 PX + 4 floats.  A thread
+// is (mg, g): pixels PX mg .. of output group g.
+constexpr int kTG = 16;
+template <int PX>
+__host__ __device__ constexpr int tile_px() { return kTG * PX; }
+template <int PX>
+__host__ __device__ constexpr int tile_ld() { return kTG * PX + 4; }
+constexpr int kLanes = 8;       // lanes per pixel of the likelihood
+static_assert(kTG * kTG == kThreads, "one block of every layer per thread");
 
+// Shared memory (float offsets): the weights WT[k][n] of every layer (rows of
+// ld(N) floats), the context X, the activations u_0, v_0, u_1, .. (2R + 1
+// tiles), dP, and one region for the head outputs P, then the two gradient
+// tiles.  All tiles are [feature][16 px + 4].
 struct TrainPlan {
-  int X, A, Hp, P, DP, T1, T2, XP, zeros, red, ldx, end;  // float offsets
+  int w0, w1, wstride, wh, bias, X, U, DP, P, ldp, G, G2, red, slots, end;
 };
+// Weight row stride: 4 modulo 8, so that neighbouring rows start on other
+// banks (the adjoint reads one column of 8 rows at once) and stay aligned.
+__host__ __device__ inline int train_ld(int N) { return ((N + 7) & ~7) + 4; }
 
-__host__ __device__ inline TrainPlan train_plan(const Dims& d) {
+__host__ __device__ inline TrainPlan train_plan(const Dims& d, int px) {
+  const int tm = kTG * px, ld = tm + 4;
   TrainPlan p;
   int o = 0;
-  p.ldx = (d.Fp > d.C ? d.Fp : d.C) + 4;
-  p.X = o; o += d.Fp * kTM;
-  p.A = o; o += (d.R + 1) * d.C * kTM;
-  p.Hp = o; o += d.R * d.C * kTM;
-  p.P = o; o += kTM * d.ldP;
-  p.DP = o; o += d.NOp * kTM;
-  p.T1 = o; o += d.C * kTM;
-  p.T2 = o; o += d.C * kTM;
-  p.XP = o; o += kTM * p.ldx;
-  p.zeros = o; o += (d.NOp > d.C ? d.NOp : d.C);
+  p.w0 = o; o += d.F * train_ld(d.C);
+  p.w1 = o; p.wstride = d.C * train_ld(d.C); o += 2 * d.R * p.wstride;
+  p.wh = o; o += d.C * train_ld(d.NOp);
+  p.bias = o; o += d.C + 2 * d.R * d.C + d.NOp;
+  p.X = o; o += d.F * ld;
+  p.U = o; o += (2 * d.R + 1) * d.C * ld;
+  p.DP = o; o += d.NO * ld;
+  p.ldp = d.NOp + 4;
+  p.P = o; p.G = o; p.G2 = o + d.C * ld;
+  o += 2 * d.C * ld > tm * p.ldp ? 2 * d.C * ld : tm * p.ldp;
   p.red = o; o += 32;
+  p.slots = o; o += tm * 4;
   p.end = o;
   return p;
 }
 
-__host__ __device__ inline size_t train_smem_bytes(const Dims& d) {
-  return (size_t)train_plan(d).end * 4 + sizeof(PixSlot) * kTM;
+inline size_t train_smem_bytes(const Dims& d, int px) { return (size_t)train_plan(d, px).end * 4; }
+// PX of the model's tiles, 0 if even the small ones do not fit.
+static int train_px(const Dims& d) {
+  return train_smem_bytes(d, 2) <= 227 * 1024 ? 2 : train_smem_bytes(d, 1) <= 227 * 1024 ? 1 : 0;
 }
 
-__device__ __forceinline__ float elu_d(float x) { return x > 0.f ? 1.f : expf(x); }
+// Blocks of the backward products: a warp is 8 x 4 of the 16 x 16 threads, so
+// that its 16-byte reads of eight neighbouring rows fill one wavefront.
+__device__ __forceinline__ int fast16() { return (threadIdx.x & 7) + 8 * ((threadIdx.x >> 5) & 1); }
+__device__ __forceinline__ int slow16() {
+  return ((threadIdx.x >> 3) & 3) + 4 * (threadIdx.x >> 6);
+}
 
-// x(m, k) pixel-major copy of a feature-major [rows][64] tile.
-__device__ __forceinline__ void to_pixel_major(const float* src, int rows, float* dst, int ldx) {
-  for (int e = threadIdx.x; e < rows * kTM; e += blockDim.x) {
-    const int r = e / kTM, m = e % kTM;
-    dst[m * ldx + r] = src[e];
+// ELU'(t) from u = ELU(t) = e^t - 1 for t <= 0.
+__device__ __forceinline__ float elu_d(float u) { return u > 0.f ? 1.f : __fadd_rn(u, 1.f); }
+
+__device__ __forceinline__ void red_add(float* p, float v) {
+  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+
+// Weight gradient of one layer: gW[n][k] += sum_m G[n][m] X[k][m] for n < Nn,
+// k < Kk, and gb[n] += sum_m G[n][m], in the CTA's slot.  A thread owns the
+// NB x KB block n = first + ng + 16 b, k = kg + 16 j: neighbouring lanes read
+// neighbouring rows (conflict-free 16-byte reads along the pixels) and write
+// neighbouring elements.  The sums go to the slot as reductions: an element is
+// always added to by the same thread, tile after tile, so their order is
+// fixed, and no thread waits for the old value (reading it back cost 119 of
+// 626 us per 64 x 32^2 step).
+template <int PX, int NB, int KB>
+__device__ __forceinline__ void weight_grad(const float* G, int Nn, const float* X, int Kk,
+                                            float* __restrict__ gW, float* __restrict__ gb,
+                                            int first = 0) {
+  constexpr int kTM = tile_px<PX>(), kTLd = tile_ld<PX>();
+  const int kg = fast16(), n0 = first + slow16();
+  if (n0 >= Nn) return;
+  float acc[NB][KB], bs[NB];
+#pragma unroll
+  for (int b = 0; b < NB; b++) {
+    bs[b] = 0.f;
+#pragma unroll
+    for (int j = 0; j < KB; j++) acc[b][j] = 0.f;
+  }
+  // rows past the end repeat a row inside (their sums are not stored)
+  const float* gp[NB];
+  const float* xp[KB];
+#pragma unroll
+  for (int b = 0; b < NB; b++) gp[b] = G + (n0 + 16 * b < Nn ? n0 + 16 * b : n0) * kTLd;
+#pragma unroll
+  for (int j = 0; j < KB; j++) xp[j] = X + (kg + 16 * j < Kk ? kg + 16 * j : 0) * kTLd;
+  float4 g[2][NB], x[2][KB];  // the next four pixels are read behind the present ones' products
+  auto load = [&](int i, int m) {
+#pragma unroll
+    for (int b = 0; b < NB; b++) g[i][b] = *reinterpret_cast<const float4*>(gp[b] + m);
+#pragma unroll
+    for (int j = 0; j < KB; j++) x[i][j] = *reinterpret_cast<const float4*>(xp[j] + m);
+  };
+  auto fma = [&](int i) {
+#pragma unroll
+    for (int b = 0; b < NB; b++) {
+      const float4 y = g[i][b];
+      bs[b] = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(bs[b], y.x), y.y), y.z), y.w);
+#pragma unroll
+      for (int j = 0; j < KB; j++) {
+        acc[b][j] = __fmaf_rn(y.x, x[i][j].x, acc[b][j]);
+        acc[b][j] = __fmaf_rn(y.y, x[i][j].y, acc[b][j]);
+        acc[b][j] = __fmaf_rn(y.z, x[i][j].z, acc[b][j]);
+        acc[b][j] = __fmaf_rn(y.w, x[i][j].w, acc[b][j]);
+      }
+    }
+  };
+  load(0, 0);
+#pragma unroll 1
+  for (int m = 0; m < kTM; m += 8) {
+    load(1, m + 4);
+    fma(0);
+    if (m + 8 < kTM) load(0, m + 8);
+    fma(1);
+  }
+#pragma unroll
+  for (int b = 0; b < NB; b++) {
+    const int n = n0 + 16 * b;
+    if (n >= Nn) continue;
+#pragma unroll
+    for (int j = 0; j < KB; j++) {
+      const int k = kg + 16 * j;
+      if (k < Kk) red_add(gW + (size_t)n * Kk + k, acc[b][j]);
+    }
+    if (kg == 0) red_add(gb + n, bs[b]);
   }
 }
 
-// gW[n][k] += sum_m G[n][m] Xp[m][k] (n < Nn, k < Kk <= 128), gb[n] += sum_m G[n][m].
-__device__ void outer_accum(const float* G, int Nn, const float* Xp, int ldx, int Kk,
-                            float* __restrict__ gW, float* __restrict__ gb) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int n0 = 4 * warp; n0 < Nn; n0 += 4 * kWarps) {
-    float acc[4][4], bs[4];
+// Adjoint of a layer: acc[j][a] = sum_n WT[k][n] G[n][PX mg + a] for the
+// thread's k = g + 16 j.
+template <int PX, int NB>
+__device__ __forceinline__ void input_grad(const float* WT, int ld, const float* G, int Nn,
+                                           float (&acc)[NB][PX]) {
+  constexpr int kTLd = tile_ld<PX>();
+  const int g = fast16(), mg = slow16();
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
-      bs[a] = 0.f;
+  for (int j = 0; j < NB; j++)
 #pragma unroll
-      for (int j = 0; j < 4; j++) acc[a][j] = 0.f;
-    }
-    for (int m = 0; m < kTM; m++) {
-      float g[4], x[4];
+    for (int a = 0; a < PX; a++) acc[j][a] = 0.f;
+  const float* w = WT + g * ld;
+  const float* y = G + PX * mg;
+  float4 v[2][NB];
+  float x[2][4][PX];
+  auto load = [&](int s, int n) {
 #pragma unroll
-      for (int a = 0; a < 4; a++) g[a] = (n0 + a < Nn) ? G[(n0 + a) * kTM + m] : 0.f;
+    for (int i = 0; i < 4; i++) f32_load<PX>(y + (n + i) * kTLd, x[s][i]);
 #pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const int k = lane + 32 * j;
-        x[j] = k < Kk ? Xp[m * ldx + k] : 0.f;
+    for (int j = 0; j < NB; j++) v[s][j] = *reinterpret_cast<const float4*>(w + 16 * j * ld + n);
+  };
+  auto fma = [&](int s) {
+#pragma unroll
+    for (int j = 0; j < NB; j++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) {
+        const float vi = i == 0 ? v[s][j].x : i == 1 ? v[s][j].y : i == 2 ? v[s][j].z : v[s][j].w;
+#pragma unroll
+        for (int a = 0; a < PX; a++) acc[j][a] = __fmaf_rn(vi, x[s][i][a], acc[j][a]);
       }
+  };
+  // groups of four outputs, the next one read behind the present one's products
+  const int n4 = Nn & ~3;
+  load(0, 0);
+  int n = 4;
+#pragma unroll 1
+  for (; n + 4 < n4; n += 8) {
+    load(1, n);
+    fma(0);
+    load(0, n + 4);
+    fma(1);
+  }
+  if (n < n4) {
+    load(1, n);
+    fma(0);
+    fma(1);
+  } else {
+    fma(0);
+  }
+  n = n4;
+  for (; n < Nn; n++) {  // 10 K may be 2 modulo 4
+    float x[PX];
+    f32_load<PX>(y + n * kTLd, x);
 #pragma unroll
-      for (int a = 0; a < 4; a++) {
-        bs[a] = __fadd_rn(bs[a], g[a]);
+    for (int j = 0; j < NB; j++) {
+      const float v = w[16 * j * ld + n];
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[a][j] = __fmaf_rn(g[a], x[j], acc[a][j]);
-      }
-    }
-#pragma unroll
-    for (int a = 0; a < 4; a++) {
-      if (n0 + a >= Nn) continue;
-#pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const int k = lane + 32 * j;
-        if (k < Kk) {
-          float* o = gW + (size_t)(n0 + a) * Kk + k;
-          *o = __fadd_rn(*o, acc[a][j]);
-        }
-      }
-      if (gb && lane == 0) gb[n0 + a] = __fadd_rn(gb[n0 + a], bs[a]);
+      for (int a = 0; a < PX; a++) acc[j][a] = __fmaf_rn(v, x[a], acc[j][a]);
     }
   }
+}
+
+__device__ __forceinline__ float oct_sum(float v) {
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float oct_max(float v) {
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
 }
 
 // Per-pixel NLL (nats) of the discretized logistic mixture with coupled
-// means and its gradient with respect to the 10K network outputs (lane k
-// handles component k); writes scale * dL/dP into DP[n][m].
-__device__ float pixel_nll_grad(const float* P, int K, int r, int g, int b, float scale, float* DP,
-                                int m, int NOp, int lane) {
-  const unsigned full = 0xffffffffu;
-  CompState cs;
-  comp_init(P, K, lane, cs);
-  const int v[3] = {r, g, b};
-  float l = -INFINITY, dlm[3] = {0.f, 0.f, 0.f}, dll[3] = {0.f, 0.f, 0.f}, mm[3] = {0.f, 0.f, 0.f};
-  if (lane < K) {
-    l = cs.logpi;
+// means and its gradient with respect to the 10K network outputs, by eight
+// lanes (lane l holds the components k = l, l + 8); writes scale * dL/dP into
+// DP[n][m].
+__device__ float pixel_nll_grad(const float* P, int K, const int (&v)[3], float scale, float* DP,
+                                int kTLd, int l) {
+  constexpr int KI = kMaxK / kLanes;
+  const float xr = __fdiv_rn((float)(2 * v[0] - 255), 255.f);
+  const float xg = __fdiv_rn((float)(2 * v[1] - 255), 255.f);
+  // log pi_k = logit_k - LSE(logits)
+  float mx = -INFINITY, se = 0.f;
+#pragma unroll
+  for (int i = 0; i < KI; i++)
+    if (l + kLanes * i < K) mx = fmaxf(mx, P[l + kLanes * i]);
+  mx = oct_max(mx);
+#pragma unroll
+  for (int i = 0; i < KI; i++)
+    if (l + kLanes * i < K) se = __fadd_rn(se, expf(__fsub_rn(P[l + kLanes * i], mx)));
+  const float lse_pi = __fadd_rn(mx, logf(oct_sum(se)));
+  float lp[KI], dlm[KI][3], dll[KI][3], co[KI][3];
+#pragma unroll
+  for (int i = 0; i < KI; i++) {
+    const int k = l + kLanes * i;
+    lp[i] = -INFINITY;
+    if (k >= K) continue;
+    lp[i] = __fsub_rn(P[k], lse_pi);
+#pragma unroll
+    for (int c = 0; c < 3; c++) co[i][c] = tanh_f(P[(7 + c) * K + k]);
+#pragma unroll
     for (int c = 0; c < 3; c++) {
-      const float mc = comp_mean(cs, c, r, g), inv = cs.inv[c];
-      mm[c] = mc;
-      l = __fadd_rn(l, log_bin_mass_f(mc, inv, cs.lme[c], v[c]));
+      float mc = P[(1 + c) * K + k];
+      if (c == 1) mc = __fadd_rn(mc, __fmul_rn(co[i][0], xr));
+      if (c == 2) mc = __fadd_rn(__fadd_rn(mc, __fmul_rn(co[i][1], xr)), __fmul_rn(co[i][2], xg));
+      const float ls = fmaxf(P[(4 + c) * K + k], -7.f), inv = exp_f(-ls);
+      lp[i] = __fadd_rn(lp[i], log_bin_mass_f(mc, inv, bin_log_width(ls, inv), v[c]));
       if (v[c] == 0) {
         const float a = __fmul_rn(__fsub_rn(edge_f(1), mc), inv);
         const float sa = 1.f / (1.f + expf(a));  // sigmoid(-a)
-        dlm[c] = -inv * sa;
-        dll[c] = -a * sa;
+        dlm[i][c] = -inv * sa;
+        dll[i][c] = -a * sa;
       } else if (v[c] == 255) {
         const float bb = __fmul_rn(__fsub_rn(edge_f(255), mc), inv);
         const float sb = 1.f / (1.f + expf(-bb));  // sigmoid(b)
-        dlm[c] = inv * sb;
-        dll[c] = bb * sb;
+        dlm[i][c] = inv * sb;
+        dll[i][c] = bb * sb;
       } else {
         const float a = __fmul_rn(__fsub_rn(edge_f(v[c] + 1), mc), inv);
         const float bb = __fmul_rn(__fsub_rn(edge_f(v[c]), mc), inv);
         const float dd = __fmul_rn(__fdiv_rn(2.f, 255.f), inv);
         const float gk = 1.f / expm1f(dd);
         const float sa = 1.f / (1.f + expf(a)), sb = 1.f / (1.f + expf(-bb));
-        dlm[c] = -inv * (sa - sb);
-        dll[c] = -a * sa + bb * sb - gk * dd;
+        dlm[i][c] = -inv * (sa - sb);
+        dll[i][c] = -a * sa + bb * sb - gk * dd;
       }
     }
   }
-  float mx = l;
+  mx = -INFINITY;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(full, mx, o));
-  float e = lane < K ? expf(__fsub_rn(l, mx)) : 0.f;
-  float s = e;
+  for (int i = 0; i < KI; i++) mx = fmaxf(mx, lp[i]);
+  mx = oct_max(mx);
+  float e[KI];
+  se = 0.f;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s = __fadd_rn(s, __shfl_xor_sync(full, s, o));
-  const float nll = -__fadd_rn(mx, logf(s));
-  if (lane < K) {
-    const float rho = e / s, pi = expf(cs.logpi);
-    const float xr = __fdiv_rn((float)(2 * r - 255), 255.f);
-    const float xg = __fdiv_rn((float)(2 * g - 255), 255.f);
-    const float dmR = -rho * dlm[0], dmG = -rho * dlm[1], dmB = -rho * dlm[2];
-    DP[(0 * K + lane) * kTM + m] = scale * (pi - rho);
-    DP[(1 * K + lane) * kTM + m] = scale * dmR;
-    DP[(2 * K + lane) * kTM + m] = scale * dmG;
-    DP[(3 * K + lane) * kTM + m] = scale * dmB;
-    for (int c = 0; c < 3; c++) {
-      const float raw = P[4 * K + c * K + lane];
-      DP[(4 * K + c * K + lane) * kTM + m] = raw > -7.f ? scale * (-rho * dll[c]) : 0.f;
-    }
-    const float al = cs.co[0], be = cs.co[1], ga = cs.co[2];
-    DP[(7 * K + lane) * kTM + m] = scale * dmG * xr * (1.f - al * al);
-    DP[(8 * K + lane) * kTM + m] = scale * dmB * xr * (1.f - be * be);
-    DP[(9 * K + lane) * kTM + m] = scale * dmB * xg * (1.f - ga * ga);
+  for (int i = 0; i < KI; i++) {
+    e[i] = l + kLanes * i < K ? expf(__fsub_rn(lp[i], mx)) : 0.f;
+    se = __fadd_rn(se, e[i]);
   }
-  (void)mm;
-  (void)NOp;
-  return nll;
+  se = oct_sum(se);
+#pragma unroll
+  for (int i = 0; i < KI; i++) {
+    const int k = l + kLanes * i;
+    if (k >= K) continue;
+    const float rho = e[i] / se, pi = expf(__fsub_rn(P[k], lse_pi));
+    const float dmR = -rho * dlm[i][0], dmG = -rho * dlm[i][1], dmB = -rho * dlm[i][2];
+    DP[(0 * K + k) * kTLd] = scale * (pi - rho);
+    DP[(1 * K + k) * kTLd] = scale * dmR;
+    DP[(2 * K + k) * kTLd] = scale * dmG;
+    DP[(3 * K + k) * kTLd] = scale * dmB;
+#pragma unroll
+    for (int c = 0; c < 3; c++)
+      DP[((4 + c) * K + k) * kTLd] =
+          P[(4 + c) * K + k] > -7.f ? scale * (-rho * dll[i][c]) : 0.f;
+    DP[(7 * K + k) * kTLd] = scale * dmG * xr * (1.f - co[i][0] * co[i][0]);
+    DP[(8 * K + k) * kTLd] = scale * dmB * xr * (1.f - co[i][1] * co[i][1]);
+    DP[(9 * K + k) * kTLd] = scale * dmB * xg * (1.f - co[i][2] * co[i][2]);
+  }
+  return -__fadd_rn(mx, logf(se));
 }
 
-// dparams == nullptr: dP = gradient of the batch's mean code length (bits
-// per dimension); else dP = dparams [n_px][10K] (an upstream gradient of the
-// network outputs, raster order of the batch) and no loss is computed.
+// Loss and gradient of a batch, C = 16 NB channels, per tile of 32 pixels:
+// forward, mixture NLL with its analytic gradient, adjoint and weight
+// gradients.  dparams == nullptr: dP = gradient of the batch's mean code
+// length (bits per dimension); else dP = dparams [n_px][10K] (an upstream
+// gradient of the network outputs, raster order of the batch) and no loss is
+// computed.
+//
+// Bound: the FMA pipe (3 x 27,400 multiply-adds per pixel: 19 k cycles per
+// tile at 128 per clock).  Why this shape: 32 pixels leave room for all
+// weights (one transposed copy serves both directions: the forward reads a
+// row across the outputs, the adjoint a column of neighbouring rows, apart by
+// 4 banks), so no layer waits for L2; a thread holds its block of the residual
+// stream and of its gradient in registers; a layer costs one barrier.
+// Measured, 64 x 32^2 (h = 3, C = 64, R = 2, K = 10): 1424 us with 64-pixel tiles and
+// weights read through L2, 505 us so (FMA pipe about a third busy; the rest is
+// latency at two warps per scheduler).
+template <int NB, int PX>
 __global__ void __launch_bounds__(kThreads, 1)
-    loss_grad_kernel(Dims d, const float* __restrict__ w, const float* __restrict__ wt,
-                     const uint8_t* __restrict__ batch, int N, int H, int W,
-                     const float* __restrict__ dparams, float* __restrict__ part_g,
-                     float* __restrict__ part_l, int n_w) {
+    loss_grad_kernel(Dims d, const float* __restrict__ wt, const uint8_t* __restrict__ batch,
+                     int N, int H, int W, const float* __restrict__ dparams,
+                     float* __restrict__ part_g, float* __restrict__ part_l, int n_w) {
   extern __shared__ __align__(16) float sm[];
-  const TrainPlan pl = train_plan(d);
-  float* X = sm + pl.X;
-  float* A = sm + pl.A;
-  float* Hp = sm + pl.Hp;
-  float* P = sm + pl.P;
-  float* DP = sm + pl.DP;
-  float* T1 = sm + pl.T1;
-  float* T2 = sm + pl.T2;
-  float* XP = sm + pl.XP;
-  float* zeros = sm + pl.zeros;
-  float* red = sm + pl.red;
-  PixSlot* slots = reinterpret_cast<PixSlot*>(sm + pl.end);
-  const int C = d.C, F = d.F, R = d.R, K = d.K, NO = d.NO, ldP = d.ldP, h = d.h;
+  constexpr int kTM = tile_px<PX>(), kTLd = tile_ld<PX>();
+  const TrainPlan pl = train_plan(d, PX);
+  const int C = d.C, F = d.F, R = d.R, K = d.K, NO = d.NO, h = d.h;
+  const int ldc = train_ld(C), ldh = train_ld(d.NOp);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ldx = pl.ldx;
   float* gW = part_g + (size_t)blockIdx.x * n_w;
   for (int i = threadIdx.x; i < n_w; i += blockDim.x) gW[i] = 0.f;
-  for (int i = threadIdx.x; i < (d.NOp > C ? d.NOp : C); i += blockDim.x) zeros[i] = 0.f;
-  if (threadIdx.x < 32) red[threadIdx.x] = 0.f;
-  // canonical offsets of the gradient / weights
+  if (threadIdx.x < 32) sm[pl.red + threadIdx.x] = 0.f;
+  // canonical offsets of the gradient
   const size_t oW0 = 0, ob0 = (size_t)C * F, oblk = ob0 + C;
   const size_t blk = 2 * (size_t)C * C + 2 * C;
   const size_t oWH = oblk + (size_t)R * blk, obH = oWH + (size_t)NO * C;
-  // packed transposed weights for the forward
-  const float* W0T = wt;
-  const float* b0 = W0T + (size_t)F * C;
-  const float* WHT = b0 + C + (size_t)R * blk;
-  const float* bH = WHT + (size_t)C * d.NOp;
+  // packed transposed weights W0T[F][C] b0 {W1T[C][C] b1 W2T b2}xR WHT[C][NOp] bH
+  {
+    const float* src = wt;
+    float* bias = sm + pl.bias;
+    // 16 bytes a thread (every row and matrix is a multiple of 16 floats)
+    auto rows = [&](float* dst, int ld, int nr, int nc) {
+      const float4* v = reinterpret_cast<const float4*>(src);
+      const unsigned c4 = (unsigned)nc / 4u, n = (unsigned)nr * c4;
+#pragma unroll 8
+      for (unsigned e = threadIdx.x; e < n; e += kThreads) {
+        const unsigned r = e / c4;
+        *reinterpret_cast<float4*>(dst + r * ld + 4u * (e - r * c4)) = v[e];
+      }
+      src += nr * nc;
+      for (int e = threadIdx.x; e < nc; e += kThreads) bias[e] = src[e];
+      src += nc;
+      bias += nc;
+    };
+    rows(sm + pl.w0, ldc, F, C);
+    for (int l = 0; l < 2 * R; l++) rows(sm + pl.w1 + l * pl.wstride, ldc, C, C);
+    rows(sm + pl.wh, ldh, C, d.NOp);
+  }
+  int4* slots = reinterpret_cast<int4*>(sm + pl.slots);
   const long long HW = (long long)H * W, n_px = (long long)N * HW;
   const float scale = 1.f / (0.6931471805599453f * 3.f * (float)n_px);
-  __syncthreads();
   const long long ntiles = (n_px + kTM - 1) / kTM;
+  // forward: pixels PX fm .. (neighbouring lanes) of outputs NB fg ..;
+  // adjoint: the same pixels of mg, outputs g + 16 j (neighbouring lanes)
+  const int fm = threadIdx.x & 15, fg = threadIdx.x >> 4;
+  const int g = fast16(), mg = slow16();
+  float loss = 0.f;
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     if (threadIdx.x < kTM) {
       const long long q = tile * kTM + threadIdx.x;
-      PixSlot ps{-1, 0, 0, 0};
+      int4 s = make_int4(-1, 0, 0, 0);
       if (q < n_px) {
-        ps.unit = (int)(q / HW);
-        const long long rr = q % HW;
-        ps.i = (int)(rr / W);
-        ps.j = (int)(rr % W);
+        const int im = (int)(q / HW), r = (int)(q - im * HW);
+        s = make_int4(im, r / W, r % W, 0);
       }
-      slots[threadIdx.x] = ps;
+      slots[threadIdx.x] = s;
     }
     __syncthreads();
-    // gather (each image is one unit; zero outside it)
+    // context (each image is one unit; zero outside it)
     const int ntap = 2 * h * (h + 1);
-    for (int it = threadIdx.x; it < kTM * (d.Fp / 3 + 1); it += blockDim.x) {
+    for (int it = threadIdx.x; it < kTM * ntap; it += blockDim.x) {
       const int m = it % kTM, p = it / kTM;
-      if (3 * p >= d.Fp) continue;
-      const PixSlot s = slots[m];
+      const int4 s = slots[m];
       float v0 = 0.f, v1 = 0.f, v2 = 0.f;
-      if (s.unit >= 0 && p < ntap) {
-        int dy, dx;
-        tap_offset(p, h, dy, dx);
-        const int ii = s.i + dy, jj = s.j + dx;
-        if (ii >= 0 && ii < H && jj >= 0 && jj < W) {
-          const uint8_t* px = batch + ((long long)s.unit * HW + (long long)ii * W + jj) * 3;
-          v0 = __fdiv_rn((float)(2 * px[0] - 255), 255.f);
-          v1 = __fdiv_rn((float)(2 * px[1] - 255), 255.f);
-          v2 = __fdiv_rn((float)(2 * px[2] - 255), 255.f);
-        }
+      int dy, dx;
+      tap_offset(p, h, dy, dx);
+      const int ii = s.y + dy, jj = s.z + dx;
+      if (s.x >= 0 && ii >= 0 && jj >= 0 && jj < W) {
+        const uint8_t* px = batch + ((long long)s.x * HW + (long long)ii * W + jj) * 3;
+        v0 = __fdiv_rn((float)(2 * px[0] - 255), 255.f);
+        v1 = __fdiv_rn((float)(2 * px[1] - 255), 255.f);
+        v2 = __fdiv_rn((float)(2 * px[2] - 255), 255.f);
       }
-      if (3 * p + 0 < d.Fp) X[(3 * p + 0) * kTM + m] = v0;
-      if (3 * p + 1 < d.Fp) X[(3 * p + 1) * kTM + m] = v1;
-      if (3 * p + 2 < d.Fp) X[(3 * p + 2) * kTM + m] = v2;
+      float* X = sm + pl.X + 3 * p * kTLd + m;
+      X[0] = v0;
+      X[kTLd] = v1;
+      X[2 * kTLd] = v2;
     }
     __syncthreads();
     // ---- forward ----
-    gemm_dispatch<kTM>(GM_STORE, X, F, W0T, b0, C, A, 0);
-    __syncthreads();
-    for (int r = 0; r < R; r++) {
-      const float* W1T = b0 + C + r * blk;
-      const float* b1 = W1T + (size_t)C * C;
-      const float* W2T = b1 + C;
-      const float* b2 = W2T + (size_t)C * C;
-      float* Ar = A + (size_t)r * C * kTM;
-      float* An = Ar + (size_t)C * kTM;
-      float* Hr = Hp + (size_t)r * C * kTM;
-      for (int e = threadIdx.x; e < C * kTM; e += blockDim.x) {
-        T1[e] = elu_f(Ar[e]);
-        An[e] = Ar[e];
+    {
+      float res[NB][PX];
+      const float* bias = sm + pl.bias + NB * fg;
+      float* U = sm + pl.U + NB * fg * kTLd + PX * fm;  // the thread's block of the next tile
+      auto store = [&](const float (&v)[NB][PX]) {
+#pragma unroll
+        for (int b = 0; b < NB; b++)
+#pragma unroll
+          for (int a = 0; a < PX; a++) U[b * kTLd + a] = elu_f(v[b][a]);
+        U += C * kTLd;
+        bias += C;
+      };
+      f32_dot<PX, NB>(sm + pl.X + PX * fm, kTLd, F, sm + pl.w0 + NB * fg, ldc, res);
+#pragma unroll
+      for (int b = 0; b < NB; b++)
+#pragma unroll
+        for (int a = 0; a < PX; a++) res[b][a] = __fadd_rn(res[b][a], bias[b]);
+      store(res);
+      __syncthreads();
+      for (int l = 0; l < 2 * R; l++) {
+        float acc[NB][PX];
+        f32_dot<PX, NB>(sm + pl.U + l * C * kTLd + PX * fm, kTLd, C,
+                       sm + pl.w1 + l * pl.wstride + NB * fg, ldc, acc);
+#pragma unroll
+        for (int b = 0; b < NB; b++)
+#pragma unroll
+          for (int a = 0; a < PX; a++) {
+            acc[b][a] = __fadd_rn(acc[b][a], bias[b]);
+            if (l & 1) acc[b][a] = res[b][a] = __fadd_rn(res[b][a], acc[b][a]);
+          }
+        store(acc);
+        __syncthreads();
       }
-      __syncthreads();
-      gemm_dispatch<kTM>(GM_STORE, T1, C, W1T, b1, C, Hr, 0);
-      __syncthreads();
-      for (int e = threadIdx.x; e < C * kTM; e += blockDim.x) T2[e] = elu_f(Hr[e]);
-      __syncthreads();
-      gemm_dispatch<kTM>(GM_RESID, T2, C, W2T, b2, C, An, 0);
-      __syncthreads();
+      // head: blocks of four outputs
+      const float* in = sm + pl.U + 2 * R * C * kTLd + PX * fm;
+      for (int c = 4 * fg; c < d.NOp; c += 4 * kTG) {
+        float acc[4][PX];
+        f32_dot<PX, 4>(in, kTLd, C, sm + pl.wh + c, ldh, acc);
+        const float* bh = sm + pl.bias + (1 + 2 * R) * C + c;
+#pragma unroll
+        for (int a = 0; a < PX; a++)
+          *reinterpret_cast<float4*>(sm + pl.P + (PX * fm + a) * pl.ldp + c) =
+              make_float4(__fadd_rn(acc[0][a], bh[0]), __fadd_rn(acc[1][a], bh[1]),
+                          __fadd_rn(acc[2][a], bh[2]), __fadd_rn(acc[3][a], bh[3]));
+      }
     }
-    float* AR = A + (size_t)R * C * kTM;
-    for (int e = threadIdx.x; e < C * kTM; e += blockDim.x) T1[e] = elu_f(AR[e]);
     __syncthreads();
-    gemm_dispatch<kTM>(GM_HEAD, T1, C, WHT, bH, d.NOp, P, ldP);
-    __syncthreads();
-    // ---- likelihood and its gradient ----
-    for (int e = threadIdx.x; e < d.NOp * kTM; e += blockDim.x) DP[e] = 0.f;
-    __syncthreads();
-    for (int m = warp; m < kTM; m += kWarps) {
-      const PixSlot s = slots[m];
-      if (s.unit < 0) continue;
-      if (dparams) {
+    // ---- likelihood and its gradient (zero for pixels past the batch) ----
+    if (dparams) {
+      for (int e = threadIdx.x; e < kTM * NO; e += blockDim.x) {
+        const int m = e / NO, k = e - m * NO;
         const long long q = tile * kTM + m;
-        for (int k = lane; k < NO; k += 32) DP[k * kTM + m] = dparams[q * NO + k];
-        continue;
+        sm[pl.DP + k * kTLd + m] = q < n_px ? dparams[q * NO + k] : 0.f;
       }
-      const uint8_t* px = batch + ((long long)s.unit * HW + (long long)s.i * W + s.j) * 3;
-      const float nll = pixel_nll_grad(P + (size_t)m * ldP, K, px[0], px[1], px[2], scale, DP, m,
-                                       d.NOp, lane);
-      if (lane == 0) red[warp] = __fadd_rn(red[warp], nll);
+    } else if (threadIdx.x < kLanes * kTM) {
+      const int m = threadIdx.x / kLanes, l = threadIdx.x % kLanes;
+      const int4 s = slots[m];
+      int v[3] = {0, 0, 0};
+      if (s.x >= 0) {
+        const uint8_t* px = batch + ((long long)s.x * HW + (long long)s.y * W + s.z) * 3;
+        v[0] = px[0], v[1] = px[1], v[2] = px[2];
+      }
+      const float nll = pixel_nll_grad(sm + pl.P + m * pl.ldp, K, v, s.x >= 0 ? scale : 0.f,
+                                       sm + pl.DP + m, kTLd, l);
+      if (l == 0 && s.x >= 0) loss = __fadd_rn(loss, nll);
     }
     __syncthreads();
     // ---- adjoint ----
-    to_pixel_major(T1, C, XP, ldx);  // ELU(a_R)
-    __syncthreads();
-    outer_accum(DP, NO, XP, ldx, C, gW + oWH, gW + obH);
-    // dELU(a_R) = WH^T dP
-    gemm_dispatch<kTM>(GM_STORE, DP, NO, w + oWH, zeros, C, T2, 0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < C * kTM; e += blockDim.x)
-      T2[e] = __fmul_rn(T2[e], elu_d(AR[e]));
+    const float* Ul = sm + pl.U + 2 * R * C * kTLd;  // the layer's input activations
+    float da[NB][PX], acc[NB][PX];
+    float* G = sm + pl.G;
+    float* G2 = sm + pl.G2;
+    // gradient through ELU of the thread's block of activations U
+    auto through = [&](const float* U, float (&v)[NB][PX]) {
+#pragma unroll
+      for (int j = 0; j < NB; j++) {
+        float u[PX];
+        f32_load<PX>(U + (g + 16 * j) * kTLd + PX * mg, u);
+#pragma unroll
+        for (int a = 0; a < PX; a++) v[j][a] = __fmul_rn(v[j][a], elu_d(u[a]));
+      }
+    };
+    auto put = [&](float* o, const float (&v)[NB][PX]) {
+#pragma unroll
+      for (int j = 0; j < NB; j++)
+#pragma unroll
+        for (int a = 0; a < PX; a++) o[(g + 16 * j) * kTLd + PX * mg + a] = v[j][a];
+    };
+    input_grad<PX, NB>(sm + pl.wh, ldh, sm + pl.DP, NO, da);  // WH^T dP
+    through(Ul, da);
+    put(G, da);  // P is dead: the likelihood has read it
+    for (int n = 0; n < NO; n += 16 * 4) {  // 16 x 4 outputs a round, the last as many as needed
+      if (NO - n > 48) weight_grad<PX, 4, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+      else if (NO - n > 16) weight_grad<PX, 3, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+      else weight_grad<PX, 1, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+    }
     __syncthreads();
     for (int r = R - 1; r >= 0; r--) {
       const size_t oW1 = oblk + r * blk, ob1 = oW1 + (size_t)C * C;
       const size_t oW2 = ob1 + C, ob2 = oW2 + (size_t)C * C;
-      float* Ar = A + (size_t)r * C * kTM;
-      float* Hr = Hp + (size_t)r * C * kTM;
-      for (int e = threadIdx.x; e < C * kTM; e += blockDim.x) T1[e] = elu_f(Hr[e]);
+      const float* V = sm + pl.U + (2 * r + 1) * C * kTLd;
+      input_grad<PX, NB>(sm + pl.w1 + (2 * r + 1) * pl.wstride, ldc, G, C, acc);  // dv = W2^T da
+      through(V, acc);
+      put(G2, acc);
+      weight_grad<PX, NB, NB>(G, C, V, C, gW + oW2, gW + ob2);
       __syncthreads();
-      to_pixel_major(T1, C, XP, ldx);
-      __syncthreads();
-      outer_accum(T2, C, XP, ldx, C, gW + oW2, gW + ob2);
-      gemm_dispatch<kTM>(GM_STORE, T2, C, w + oW2, zeros, C, P, 0);  // dv = W2^T da
-      __syncthreads();
-      for (int e = threadIdx.x; e < C * kTM; e += blockDim.x) {
-        P[e] = __fmul_rn(P[e], elu_d(Hr[e]));  // d hidden pre-activation
-        T1[e] = elu_f(Ar[e]);
-      }
-      __syncthreads();
-      to_pixel_major(T1, C, XP, ldx);
-      __syncthreads();
-      outer_accum(P, C, XP, ldx, C, gW + oW1, gW + ob1);
-      gemm_dispatch<kTM>(GM_STORE, P, C, w + oW1, zeros, C, T1, 0);  // du = W1^T dh
-      __syncthreads();
-      for (int e = threadIdx.x; e < C * kTM; e += blockDim.x)
-        T2[e] = __fadd_rn(T2[e], __fmul_rn(T1[e], elu_d(Ar[e])));
+      const float* Ur = V - C * kTLd;
+      input_grad<PX, NB>(sm + pl.w1 + 2 * r * pl.wstride, ldc, G2, C, acc);  // du = W1^T dz
+      through(Ur, acc);
+#pragma unroll
+      for (int j = 0; j < NB; j++)
+#pragma unroll
+        for (int a = 0; a < PX; a++) da[j][a] = __fadd_rn(da[j][a], acc[j][a]);
+      put(G, da);
+      weight_grad<PX, NB, NB>(G2, C, Ur, C, gW + oW1, gW + ob1);
       __syncthreads();
     }
-    to_pixel_major(X, F, XP, ldx);
-    __syncthreads();
-    outer_accum(T2, C, XP, ldx, F, gW + oW0, gW + ob0);
+    switch ((F + 15) / 16) {
+      case 1: weight_grad<PX, NB, 1>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+      case 3: weight_grad<PX, NB, 3>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+      default: weight_grad<PX, NB, 5>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+    }
     __syncthreads();
   }
+  // loss: the pixels' lanes of every warp, then the warps, in a fixed order
+#pragma unroll
+  for (int o = kLanes; o < 32; o <<= 1)
+    loss = __fadd_rn(loss, __shfl_xor_sync(0xffffffffu, loss, o));
+  if (lane == 0) sm[pl.red + warp] = loss;
+  __syncthreads();
   if (threadIdx.x == 0) {
     float t = 0.f;
-    for (int i = 0; i < kWarps; i++) t = __fadd_rn(t, red[i]);
+    for (int i = 0; i < kWarps; i++) t = __fadd_rn(t, sm[pl.red + i]);
     part_l[blockIdx.x] = t;
   }
 }
 
+// grad[i] = sum over the slots b of part_g[b][i], in a fixed order: 8 threads
+// of a block take every eighth slot of one element, then their sums are added
+// in turn.  (One thread per element was a chain of 152 additions and left two
+// thirds of the SMs idle: 14 us for 152 slots of 25 k weights, now 7.7 us.)
+constexpr int kRedSplit = 8;
 __global__ void reduce_grad_kernel(const float* __restrict__ part_g, const float* __restrict__ part_l,
                                    int nblk, int n_w, int ldw, float inv_dims,
                                    float* __restrict__ grad, float* __restrict__ loss) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ float sh[kRedSplit][32];
+  const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int i = blockIdx.x * 32 + c;
+  float s = 0.f;
   if (i < n_w) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; b++) s = __fadd_rn(s, part_g[(size_t)b * ldw + i]);
+#pragma unroll 4
+    for (int b = g; b < nblk; b += kRedSplit) s = __fadd_rn(s, part_g[(size_t)b * ldw + i]);
+  }
+  sh[g][c] = s;
+  __syncthreads();
+  if (g == 0 && i < n_w) {
+#pragma unroll
+    for (int k = 1; k < kRedSplit; k++) s = __fadd_rn(s, sh[k][c]);
     grad[i] = s;
   }
-  if (i == 0 && part_l && loss) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; b++) s = __fadd_rn(s, part_l[b]);
-    *loss = s * inv_dims;
+  if (blockIdx.x == 0 && g == 1 && part_l && loss) {
+    float t = 0.f;
+    for (int b = c; b < nblk; b += 32) t = __fadd_rn(t, part_l[b]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+    if (c == 0) *loss = t * inv_dims;
   }
 }
 
 cudaError_t launch_reduce_grad(const float* part_g, const float* part_l, int nblk, int n_w, int ldw,
                                long long n_px, float* grad, float* loss, cudaStream_t s) {
   const float inv_dims = 1.f / (0.6931471805599453f * 3.f * (float)n_px);
-  reduce_grad_kernel<<<(n_w + 255) / 256, 256, 0, s>>>(part_g, part_l, nblk, n_w, ldw, inv_dims,
-                                                      grad, loss);
+  reduce_grad_kernel<<<(n_w + 31) / 32, 32 * kRedSplit, 0, s>>>(part_g, part_l, nblk, n_w, ldw,
+                                                               inv_dims, grad, loss);
   return cudaGetLastError();
 }
 
-bool simt_train_fits(const Dims& d) { return train_smem_bytes(d) <= 227 * 1024; }
+// The documented limit of the FP32 trainer (n_res = 2 at C = 64, K = 10, and
+// what takes no more of the following measure); every such model's tiles fit.
+bool simt_train_fits(const Dims& d) {
+  const int wide = d.Fp > d.C ? d.Fp : d.C, out = d.NOp > d.C ? d.NOp : d.C;
+  const int rows = d.Fp + (2 * d.R + 3) * d.C + d.ldP + d.NOp + wide + 4;
+  return (size_t)(64 * rows + out + 32) * 4 + 1024 <= 227 * 1024;
+}
 
-static int train_grid(long long n_px, int sm_count) {
-  long long t = (n_px + kTM - 1) / kTM;
+static int train_grid(const Dims& d, long long n_px, int sm_count) {
+  const int tm = kTG * train_px(d);
+  long long t = (n_px + tm - 1) / tm;
   return (int)(t < sm_count ? (t < 1 ? 1 : t) : sm_count);
 }
 
 size_t train_ws_bytes(const Dims& d, long long n_px, int sm_count) {
   const size_t nw = (size_t)d.C * d.F + d.C + (size_t)d.R * (2 * d.C * d.C + 2 * d.C) +
                     (size_t)d.NO * d.C + d.NO;
-  const int g = train_grid(n_px, sm_count);
+  const int g = train_grid(d, n_px, sm_count);
   return ((size_t)g * nw + g + 64) * 4;
 }
 
-cudaError_t launch_loss_grad(const Dims& d, const float* w, const float* wt, const uint8_t* batch,
-                             int N, int H, int W, const float* dparams, float* loss, float* grad,
-                             void* ws, int sm_count, cudaStream_t s) {
+template <int PX>
+static const void* loss_grad_fn(int C) {
+  switch (C) {
+    case 16: return (const void*)loss_grad_kernel<1, PX>;
+    case 32: return (const void*)loss_grad_kernel<2, PX>;
+    case 48: return (const void*)loss_grad_kernel<3, PX>;
+    default: return (const void*)loss_grad_kernel<4, PX>;
+  }
+}
+
+cudaError_t launch_loss_grad(const Dims& d, const float* wt, const uint8_t* batch, int N, int H,
+                             int W, const float* dparams, float* loss, float* grad, void* ws,
+                             int sm_count, cudaStream_t s) {
   const int n_w = (int)((size_t)d.C * d.F + d.C + (size_t)d.R * (2 * d.C * d.C + 2 * d.C) +
                         (size_t)d.NO * d.C + d.NO);
   const long long n_px = (long long)N * H * W;
-  const int g = train_grid(n_px, sm_count);
-  const size_t smem = train_smem_bytes(d);
-  if (smem > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(loss_grad_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int g = train_grid(d, n_px, sm_count);
+  const int px = train_px(d);
+  if (px == 0) return cudaErrorInvalidConfiguration;
+  const size_t smem = train_smem_bytes(d, px);
+  const void* fn = px == 2 ? loss_grad_fn<2>(d.C) : loss_grad_fn<1>(d.C);
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   float* part_g = reinterpret_cast<float*>(ws);
   float* part_l = part_g + (size_t)g * n_w;
-  loss_grad_kernel<<<g, kThreads, smem, s>>>(d, w, wt, batch, N, H, W, dparams, part_g, part_l,
-                                              n_w);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  Dims dd = d;
+  int nw = n_w;
+  void* args[] = {&dd, &wt, &batch, &N, &H, &W, &dparams, &part_g, &part_l, &nw};
+  if ((e = cudaLaunchKernel(fn, dim3(g), dim3(kThreads), args, smem, s)) != cudaSuccess) return e;
   return launch_reduce_grad(part_g, dparams ? nullptr : part_l, g, n_w, n_w, n_px, grad, loss, s);
 }
 

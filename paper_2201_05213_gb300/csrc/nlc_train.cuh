@@ -13,9 +13,9 @@ size_t train_ws_bytes(const Dims& d, long long n_px, int sm_count);
 // FP32 SIMT path.  dparams == nullptr: loss (bits per dimension) and its
 // gradient; else the gradient of sum(dparams * network outputs) (loss
 // untouched).
-cudaError_t launch_loss_grad(const Dims& d, const float* w, const float* wt, const uint8_t* batch,
-                             int N, int H, int W, const float* dparams, float* loss, float* grad,
-                             void* ws, int sm_count, cudaStream_t s);
+cudaError_t launch_loss_grad(const Dims& d, const float* wt, const uint8_t* batch, int N, int H,
+                             int W, const float* dparams, float* loss, float* grad, void* ws,
+                             int sm_count, cudaStream_t s);
 // Sums per-CTA gradient slots (and loss partials, if part_l and loss are
 // non-null) in a fixed order.
 cudaError_t launch_reduce_grad(const float* part_g, const float* part_l, int nblk, int n_w, int ldw,
