@@ -247,26 +247,4 @@ struct Front {
   int i_lo, n;  // first row and number of pixels
 };
 
-__device__ __forceinline__ Front unit_front(const Unit& u, int t, int h, int sched) {
-  Front f{0, 0};
-  int tau = t - u.start_step;
-  if (tau < 0) return f;
-  if (sched == SCHED_WAVEFRONT) {
-    int o = h + 1;
-    int hi = tau / o;
-    if (hi > u.Hu - 1) hi = u.Hu - 1;
-    int num = tau - u.Wu + 1;  // i >= ceil(num / o)
-    int lo = num <= 0 ? 0 : (num + o - 1) / o;
-    if (hi >= lo) { f.i_lo = lo; f.n = hi - lo + 1; }
-  } else {
-    if (tau < u.Hu * u.Wu) { f.i_lo = tau / u.Wu; f.n = 1; }
-  }
-  return f;
-}
-
-__device__ __forceinline__ int front_col(const Unit& u, int t, int i, int h, int sched) {
-  int tau = t - u.start_step;
-  return sched == SCHED_WAVEFRONT ? tau - (h + 1) * i : tau % u.Wu;
-}
-
 }  // namespace nlc

@@ -15,12 +15,12 @@ static int decode_threads_of(int prec) {
 // units leaves no room for 128; a share beyond one tile takes several).
 static int decode_rows(const Dims& d, int n_units, bool win) {
   if (d.prec != PREC_BF16) return kF32Rows;
-  return dec_carve(d, nullptr, n_units, kTileMax, win, nullptr) <= 227 * 1024 ? kTileMax
+  return dec_carve(d, n_units, kTileMax, win, nullptr) <= 227 * 1024 ? kTileMax
                                                                               : kTileMax / 2;
 }
 
 size_t decode_smem_bytes(const Dims& d, int n_units, bool win) {
-  return dec_carve(d, nullptr, n_units, decode_rows(d, n_units, win), win, nullptr);
+  return dec_carve(d, n_units, decode_rows(d, n_units, win), win, nullptr);
 }
 
 // The kernel for a launch; prof selects the instrumented build (decoding

@@ -43,72 +43,124 @@ struct DecodeArgs {
 template <int PREC>
 __host__ __device__ constexpr int decode_threads() { return PREC == PREC_BF16 ? 512 : kThreads; }
 
-// Shared memory of a decoder CTA.
-struct DecSmem {
-  NetSmem net;            // BF16 network
-  float* f32;             // FP32 network
-  const float* P;         // head outputs of the tile's pixels
-  int ldp;                // and their row stride
-  WarpScratch* ws;        // one per warp (whole-warp coding)
-  DecSlot* slots;         // the tile's pixels
-  StreamRec* rec;         // their stream records
-  uint32_t* win;          // per pixel, the 12 stream bytes from pos + 8, word-aligned
-  int* prow;              // sheared wavefront decoder: output row of the tile's pixel s
-  int* rofs;              // sheared wavefront decoder: ring byte offset of the tile's pixel s
-  int2* wrow;             // sheared wavefront decoder: (unit, unit row) of window row rho
-  long long* sh;
-  long long* pc;          // 16 profiling accumulators (thread 0 only)
-  int* pre;               // front prefix of the units
-  int* flag;
+// What the schedule needs of a unit.  All of them are kept in shared memory
+// when they fit: the schedule of a step is on its critical path, and each
+// dependent read of the unit table through L2 added 0.3 us to it.
+struct alignas(16) DecUnit {
+  uint8_t* px;      // first pixel
+  int Hu, Wu;       // size
+  int row_bytes;    // row stride of the image
+  int stream_base;  // first rANS stream
+  int start_step;   // step of its first pixel
+  int ring_row;     // first row in the sheared rings
 };
+__device__ __forceinline__ DecUnit dec_unit(const Unit& u) {
+  return DecUnit{u.img + ((long long)u.y0 * u.img_W + u.x0) * 3, u.Hu, u.Wu, 3 * u.img_W,
+                 u.stream_base, u.start_step, u.ring_row};
+}
+
+// x / (h + 1) for h <= 3 and x >= 0.
+__device__ __forceinline__ int div_o(int x, int h) {
+  return h == 1 ? x >> 1 : h == 3 ? x >> 2 : (int)(__umulhi((unsigned)x, 0xAAAAAAABu) >> 1);
+}
+
+// Front of a unit at global step t (see unit_front).
+__device__ __forceinline__ Front dec_front(const DecUnit& u, int t, int h, int sched) {
+  const int tau = t - u.start_step;
+  Front f{0, 0};
+  if (tau < 0) return f;
+  if (sched == SCHED_WAVEFRONT) {
+    const int hi = min(div_o(tau, h), u.Hu - 1);
+    const int num = tau - u.Wu + 1;  // i >= ceil(num / (h + 1))
+    f.i_lo = num <= 0 ? 0 : div_o(num + h, h);
+    f.n = max(hi - f.i_lo + 1, 0);
+  } else if (tau < u.Hu * u.Wu) {
+    f.i_lo = tau / u.Wu;
+    f.n = 1;
+  }
+  return f;
+}
+
+// Shared memory of a decoder CTA: byte offsets of its regions (dec_at).
+struct DecSmem {
+  int P;      // head outputs of the tile's pixels
+  int ldp;    // and their row stride
+  int ws;     // WarpScratch, one per warp (whole-warp coding)
+  int slots;  // DecSlot: the tile's pixels
+  int rec;    // StreamRec: their stream records
+  int win;    // per pixel, the 12 stream bytes from pos + 8, word-aligned (4 words)
+  int prow;   // sheared wavefront decoder: output row of the tile's pixel s
+  int rofs;   // sheared wavefront decoder: ring byte offset of the tile's pixel s
+  int wrow;   // sheared wavefront decoder: (unit, unit row) of window row rho
+  int sh;     // 33 long long: the schedule's warp sums
+  int pc;     // 16 profiling accumulators (thread 0 only)
+  int units;  // DecUnit: the batch's units, where they fit (else 0: read from global memory)
+  int pre;    // front prefix of the units
+  int flag;   // [0] stop, [1..3] sheared tile, [4], [5] units of the share, [6], [7] the share
+};
+
+// The arguments and the shared-memory map as the kernel's functions see them.
+// They are kept in shared memory: as kernel parameters and locals passed by
+// reference they were in local memory, whose lines every acquire of the grid
+// barrier drops from L1, so the first use of each field in a step went to L2.
+struct DecShared {
+  NetSmem net;
+  DecodeArgs a;
+  DecSmem t;
+};
+static_assert(sizeof(DecShared) <= kSharedHead, "the record's place");
+__device__ __forceinline__ DecShared& dec_shared() {
+  return *reinterpret_cast<DecShared*>(dec_smem);
+}
+
+constexpr size_t kMaxSmem = 227 * 1024;
 
 // Carves the shared memory of a tile of `rows` pixels; returns its bytes.
 // win: the sheared model's wavefront decoder.  The whole-warp groups' scratch
 // lies behind the first 16 head-output rows of the BF16 tile region, which a
 // tile of at most 16 pixels leaves free (not in the window tile, whose output
 // rows are spread out).
-__host__ __device__ inline size_t dec_carve(const Dims& d, unsigned char* smem, int n_pre, int rows,
-                                            bool win, DecSmem* t) {
-  size_t off;
-  unsigned char* ws;
+__host__ __device__ inline size_t dec_carve(const Dims& d, int n_pre, int rows, bool win,
+                                            DecSmem* t) {
+  int off;
   DecSmem z{};
   if (d.prec == PREC_BF16) {
     const NetPlan p = net_plan(d, rows, win);
-    off = (size_t)p.end;
-    ws = win ? smem + off : smem + p.x + kNetWarps * net_ldp(d) * 4;
-    if (win) off += sizeof(WarpScratch) * kNetWarps;
-    z.P = reinterpret_cast<const float*>(smem + p.x);
+    off = p.end;
+    z.ws = win ? off : p.x + kNetWarps * net_ldp(d) * 4;
+    if (win) off += (int)sizeof(WarpScratch) * kNetWarps;
+    z.P = p.x;
     z.ldp = net_ldp(d);
   } else {
     const F32Plan p = f32_plan(d);
-    z.f32 = reinterpret_cast<float*>(smem);
-    z.P = z.f32 + p.u;
+    z.P = 4 * p.u;
     z.ldp = d.ldP;
-    off = ((size_t)p.end * 4 + 15) & ~(size_t)15;
-    ws = smem + off;
-    off += sizeof(WarpScratch) * (decode_threads<PREC_FP32>() / 32);
+    off = align_up(p.end * 4, 16);
+    z.ws = off;
+    off += (int)sizeof(WarpScratch) * (decode_threads<PREC_FP32>() / 32);
   }
-  off = (off + 15) & ~(size_t)15;
+  off = align_up(off, 16);
   auto take = [&](size_t bytes) {
-    unsigned char* q = smem + off;
-    off += (bytes + 15) & ~(size_t)15;
-    return q;
+    const int o = off;
+    off += (int)((bytes + 15) & ~(size_t)15);
+    return o;
   };
-  z.ws = reinterpret_cast<WarpScratch*>(ws);
-  z.slots = reinterpret_cast<DecSlot*>(take(sizeof(DecSlot) * rows));
-  z.rec = reinterpret_cast<StreamRec*>(take(sizeof(StreamRec) * rows));
-  z.win = reinterpret_cast<uint32_t*>(take(4 * sizeof(uint32_t) * rows));
+  z.slots = take(sizeof(DecSlot) * rows);
+  z.rec = take(sizeof(StreamRec) * rows);
+  z.win = take(4 * sizeof(uint32_t) * rows);
   if (win) {
-    z.wrow = reinterpret_cast<int2*>(take(sizeof(int2) * (rows + 8)));
-    z.prow = reinterpret_cast<int*>(take(sizeof(int) * rows));
-    z.rofs = reinterpret_cast<int*>(take(sizeof(int) * rows));
+    z.wrow = take(sizeof(int2) * (rows + 8));
+    z.prow = take(sizeof(int) * rows);
+    z.rofs = take(sizeof(int) * rows);
   }
-  z.sh = reinterpret_cast<long long*>(take(sizeof(long long) * 33));
-  z.pc = reinterpret_cast<long long*>(take(sizeof(long long) * 16));
-  z.pre = reinterpret_cast<int*>(take(sizeof(int) * (n_pre + 1 + 4)));
-  z.flag = z.pre + n_pre + 1;
+  z.sh = take(sizeof(long long) * 33);
+  z.pc = take(sizeof(long long) * 16);
+  z.flag = take(sizeof(int) * 8);
+  z.pre = take(sizeof(int) * ((size_t)n_pre + 1));
+  if (kSharedHead + off + sizeof(DecUnit) * (size_t)n_pre <= kMaxSmem)
+    z.units = take(sizeof(DecUnit) * (size_t)n_pre);
   if (t) *t = z;
-  return off;
+  return (size_t)kSharedHead + off;
 }
 
 // Stores a decoded pixel in its unit's ring row at the byte offset rofs
@@ -144,14 +196,14 @@ __device__ __forceinline__ GroupRansDec load_rec(const StreamRec* r) {
 template <bool SAMPLE, bool SHEAR>
 __device__ __forceinline__ void put_pixel(const DecodeArgs& a, const DecSmem& t, int s,
                                           const int (&v)[3], GroupRansDec& dec) {
-  const DecSlot ps = t.slots[s];
+  const DecSlot ps = dec_at<DecSlot>(t.slots)[s];
   ps.px[0] = (uint8_t)v[0];
   ps.px[1] = (uint8_t)v[1];
   ps.px[2] = (uint8_t)v[2];
-  if (SHEAR) ring_put(a, t.rofs[s], v);
+  if (SHEAR) ring_put(a, dec_at<int>(t.rofs)[s], v);
   if (SAMPLE) return;
-  const ulonglong2 pe = *reinterpret_cast<const ulonglong2*>(&t.rec[s].pos);
-  dec.set_window(t.win + 4 * s, pe.x);
+  const ulonglong2 pe = *reinterpret_cast<const ulonglong2*>(&dec_at<StreamRec>(t.rec)[s].pos);
+  dec.set_window(dec_at<uint32_t>(t.win) + 4 * s, pe.x);
   const unsigned long long np = pe.x + (unsigned long long)dec.used;
   uint32_t n0, n1;
   dec.next_bytes(n0, n1);
@@ -194,20 +246,21 @@ struct Ticker {
 // t.rec (visible to the warp), their windows are being copied to t.win by the
 // warp's lanes.
 template <int NW, bool SAMPLE, bool SHEAR, bool PROF>
-__device__ __noinline__ void code_wide(const DecodeArgs& a, const DecSmem& t, int n,
-                                       long long* pc) {
+__device__ __noinline__ void code_wide(int n, long long* pc) {
+  const DecodeArgs& a = dec_shared().a;
+  const DecSmem& t = dec_shared().t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int K = a.m.d.K;
-  WarpScratch& ws = t.ws[warp];
+  WarpScratch& ws = dec_at<WarpScratch>(t.ws)[warp];
   Ticker<PROF> tick(pc);
   for (int s = warp; s < n; s += NW) {
     GroupRansDec dec;
     unsigned long long key = 0;
-    if (SAMPLE) key = sample_key(a, t.slots[s]);
-    else dec = load_rec(t.rec + s);
+    if (SAMPLE) key = sample_key(a, dec_at<DecSlot>(t.slots)[s]);
+    else dec = load_rec(dec_at<StreamRec>(t.rec) + s);
     if (PROF && tick.pc) tick.pc[12] += 1;
     CompState cs;
-    comp_init<32>(t.P + (size_t)(SHEAR ? t.prow[s] : s) * t.ldp, K, lane, cs);
+    comp_init<32>(dec_at<float>(t.P) + (SHEAR ? dec_at<int>(t.prow)[s] : s) * t.ldp, K, lane, cs);
     int v[3] = {0, 0, 0};
     for (int ch = 0; ch < 3; ch++) {
       int nact;
@@ -235,8 +288,9 @@ __device__ __noinline__ void code_wide(const DecodeArgs& a, const DecSmem& t, in
 // The same by quads, eight pixels per warp: warp w codes the tile's pixels
 // 8 (w + NW j) .. + 7 (see nlc_quad.cuh).
 template <int KI, int NW, bool SAMPLE, bool SHEAR, bool PROF>
-__device__ __noinline__ void code_quads(const DecodeArgs& a, const DecSmem& t, int n,
-                                        long long* pc) {
+__device__ __noinline__ void code_quads(int n, long long* pc) {
+  const DecodeArgs& a = dec_shared().a;
+  const DecSmem& t = dec_shared().t;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q = lane & 3;
   const int K = a.m.d.K;
@@ -246,10 +300,10 @@ __device__ __noinline__ void code_quads(const DecodeArgs& a, const DecSmem& t, i
     const int s = valid ? s0 + (lane >> 2) : n - 1;  // an idle quad shadows the last pixel
     GroupRansDec dec;
     unsigned long long key = 0;
-    if (SAMPLE) key = sample_key(a, t.slots[s]);
-    else dec = load_rec(t.rec + s);
+    if (SAMPLE) key = sample_key(a, dec_at<DecSlot>(t.slots)[s]);
+    else dec = load_rec(dec_at<StreamRec>(t.rec) + s);
     if (PROF && tick.pc) tick.pc[12] += 1;
-    const float* row = t.P + (size_t)(SHEAR ? t.prow[s] : s) * t.ldp + q;
+    const float* row = dec_at<float>(t.P) + (SHEAR ? dec_at<int>(t.prow)[s] : s) * t.ldp + q;
     auto P = [&](int p, int i) { return row[p * K + 4 * i]; };
     QuadState<KI> st;
     quad_init<KI>(P, K, q, st);
@@ -280,6 +334,151 @@ __device__ __noinline__ void code_quads(const DecodeArgs& a, const DecSmem& t, i
   }
 }
 
+// ---------------------------------------------------------------------
+// Schedule of a step, computed by the first nt threads of the CTA (functions
+// of their own, with their results in shared memory: inlined, their state and
+// the step loop's spilled to local memory, which the loop re-reads from L2).
+// ---------------------------------------------------------------------
+__device__ __forceinline__ DecUnit unit_of(int u) {
+  const int in = dec_shared().t.units;
+  return in ? dec_at<DecUnit>(in)[u] : dec_unit(dec_shared().a.units[u]);
+}
+
+// Fronts of all units: pre[u] = exclusive prefix of the front sizes,
+// pre[n_units] = their total F; flag[4], flag[5] = the units that hold the
+// first and the last pixel of this CTA's share [flag[6], flag[7]) of the F
+// pixels (F / grid of them, or one more).  Every warp adds up the warps' sums
+// itself: two barriers.
+static __device__ __forceinline__ void sched_front(int step, int nt) {
+  const DecodeArgs& a = dec_shared().a;
+  const DecSmem& t = dec_shared().t;
+  const int n_units = a.n_units, h = a.m.d.h, sched = a.sched;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned G = gridDim.x;
+  const int per = (n_units + nt - 1) / nt, nw = nt >> 5;
+  const int u0 = min((int)threadIdx.x * per, n_units), u1 = min(u0 + per, n_units);
+  int* pre = dec_at<int>(t.pre);
+  int* flag = dec_at<int>(t.flag);
+  int* sums = dec_at<int>(t.sh);
+  int sum = 0, c = 0;
+  for (int u = u0; u < u1; u++) {
+    c = dec_front(unit_of(u), step, h, sched).n;
+    if (per > 1) pre[u] = c;
+    sum += c;
+  }
+  int x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sums[warp] = x;
+  part_sync(nt);
+  int y = lane < nw ? sums[lane] : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int z = __shfl_up_sync(0xffffffffu, y, o);
+    if (lane >= o) y += z;
+  }
+  const int before = __shfl_sync(0xffffffffu, y, warp > 0 ? warp - 1 : 0);
+  const int F = __shfl_sync(0xffffffffu, y, 31);
+  const unsigned each = (unsigned)F / G, more = (unsigned)F - each * G;
+  const int lo = (int)(each * blockIdx.x + min(blockIdx.x, more));
+  const int hi = lo + (int)each + (blockIdx.x < more ? 1 : 0);
+  int run = x - sum + (warp > 0 ? before : 0);
+  for (int u = u0; u < u1; u++) {
+    if (per > 1) c = pre[u];
+    pre[u] = run;
+    if (run <= lo && lo < run + c) flag[4] = u;
+    if (run < hi && hi <= run + c) flag[5] = u;
+    run += c;
+  }
+  if (threadIdx.x == 0) {
+    pre[n_units] = F;
+    flag[6] = lo;
+    flag[7] = hi;
+  }
+  part_sync(nt);
+}
+
+// Slots of the tile of n pixels starting at front position base.  SHEAR: a
+// tile of at most n pixels: also their output rows prow (pixel s of the tile's
+// k-th unit piece at s + h k: each piece is preceded by h halo window rows),
+// the window rows' (unit, unit row), and flag[1..3] = the tile's pixels,
+// output rows and window rows (the output rows stay below `rows`).
+template <bool SHEAR>
+__device__ __forceinline__ void sched_slots(int step, int base, int n, int nt) {
+  const DecodeArgs& a = dec_shared().a;
+  const DecSmem& t = dec_shared().t;
+  const int h = a.m.d.h, sched = a.sched, layout = a.layout;
+  const int* pre = dec_at<int>(t.pre);
+  int* flag = dec_at<int>(t.flag);
+  DecSlot* slots = dec_at<DecSlot>(t.slots);
+  const int first = flag[4], last_u = flag[5];
+  for (int s = threadIdx.x; s < n; s += nt) {
+    const int q = base + s;
+    int lo = first, hi = last_u;  // last unit of the share with pre[u] <= q
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (pre[mid] <= q) lo = mid; else hi = mid - 1;
+    }
+    const DecUnit U = unit_of(lo);
+    const int tau = step - U.start_step;
+    DecSlot ps;
+    if (sched == SCHED_WAVEFRONT) {
+      ps.i = dec_front(U, step, h, sched).i_lo + (q - pre[lo]);
+      ps.j = tau - (h + 1) * ps.i;
+    } else {
+      ps.i = tau / U.Wu;
+      ps.j = tau - ps.i * U.Wu;
+    }
+    ps.px = U.px + (long long)ps.i * U.row_bytes + 3 * ps.j;
+    ps.Wu = U.Wu;
+    ps.row_bytes = U.row_bytes;
+    ps.stream = U.stream_base + (layout == 1 ? ps.i : 0);
+    const bool last = ps.j == U.Wu - 1 && (layout == 1 || ps.i == U.Hu - 1);
+    ps.unit = lo | (last ? (int)0x80000000 : 0);
+    if (SHEAR)  // ring bytes of the pixel's sheared column j + (h+1) i
+      dec_at<int>(t.rofs)[s] = kRingRowBytes * (U.ring_row + ps.i) + 3 * ((ps.j + (h + 1) * ps.i) & 15);
+    slots[s] = ps;
+  }
+  if (!SHEAR) return;
+  const int rows = a.rows;
+  int* sums = dec_at<int>(t.sh);
+  int2* wrow = dec_at<int2>(t.wrow);
+  part_sync(nt);
+  if ((int)threadIdx.x < rows) {  // warps 0 .. rows/32 - 1
+    const int s = threadIdx.x, w = s >> 5, l = s & 31;
+    const bool valid = s < n;
+    const int u = valid ? slots[s].unit & 0x7FFFFFFF : -1;
+    const bool start = valid && (s == 0 || u != (slots[s - 1].unit & 0x7FFFFFFF));
+    const unsigned bal = __ballot_sync(0xffffffffu, start);
+    if (l == 0) sums[w] = __popc(bal);
+    asm volatile("bar.sync 2, %0;" ::"r"(rows) : "memory");
+    int before = 0;
+    for (int k = 0; k < w; k++) before += sums[k];
+    const int seg = before + __popc(bal & (0xffffffffu >> (31 - l))) - 1;
+    const int pr = s + h * seg;
+    const bool fits = valid && pr < rows;
+    // the tile's last pixel: the next one is missing or would not fit
+    const bool valid1 = s + 1 < n;
+    const int pr1 =
+        s + 1 + h * (seg + ((valid1 && (slots[s + 1].unit & 0x7FFFFFFF) != u) ? 1 : 0));
+    dec_at<int>(t.prow)[s] = pr;
+    if (fits) {
+      const int i = slots[s].i;
+      wrow[pr + h] = make_int2(u, i);
+      if (start)
+        for (int k = 1; k <= h; k++) wrow[pr + h - k] = make_int2(i - k >= 0 ? u : -1, i - k);
+      if (!valid1 || pr1 >= rows) {
+        flag[1] = s + 1;
+        flag[2] = pr + 1;
+        flag[3] = pr + 1 + h;
+      }
+    }
+  }
+}
+
 // SHEAR: the sheared model's wavefront decoder (Section 3.1): decoded pixels
 // also go to per-unit sheared rings, and each tile's context is one window
 // tile of (unit, row) rows read from the rings, every unit's piece of the
@@ -292,125 +491,67 @@ __device__ __noinline__ void code_quads(const DecodeArgs& a, const DecSmem& t, i
 template <int PREC, bool SAMPLE, bool SHEAR, bool PROF>
 __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(DecodeArgs a) {
   constexpr int NT = decode_threads<PREC>(), NW = NT / 32;
-  extern __shared__ __align__(128) unsigned char smem[];
-  const Dims& d = a.m.d;
   const int rows = a.rows;
-  DecSmem t;
-  dec_carve(d, smem, a.n_units, rows, SHEAR, &t);
-  if constexpr (PREC == PREC_BF16) {
-    t.net = net_carve(d, smem, rows, SHEAR);
-    t.net.limit = a.mma_limit;
-    if (threadIdx.x == 0) net_setup(t.net);
-    net_load_weights(d, a.m.w, t.net);
-  } else {
-    for (int i = threadIdx.x; i < a.m.w.simt_floats; i += blockDim.x) t.f32[i] = a.m.w.simt[i];
+  const DecSmem& t = dec_shared().t;
+  uint32_t phase = 0;  // of the warp's exchanges
+  if (threadIdx.x == 0) {
+    DecShared z;
+    dec_carve(a.m.d, a.n_units, rows, SHEAR, &z.t);
+    z.a = a;
+    z.net.d = a.m.d;
+    z.net.rows = rows;
+    z.net.limit = a.mma_limit;
+    if constexpr (PREC == PREC_BF16) {
+      z.net.pl = net_plan(a.m.d, rows, SHEAR);
+      net_setup(z.net.pl);
+    }
+    dec_shared() = z;
+    dec_at<int>(z.t.flag)[0] = 0;
   }
-  if (threadIdx.x == 0) t.flag[0] = 0;
-  if (threadIdx.x < 16) t.pc[threadIdx.x] = 0;
   __syncthreads();
+  if constexpr (PREC == PREC_BF16) {
+    net_load_weights(a.m.d, a.m.w, net_smem().pl.bias);
+  } else {
+    for (int i = threadIdx.x; i < a.m.w.simt_floats; i += blockDim.x)
+      dec_at<float>(0)[i] = a.m.w.simt[i];
+  }
+  if (threadIdx.x < 16) dec_at<long long>(t.pc)[threadIdx.x] = 0;
+  if (t.units)
+    for (int u = threadIdx.x; u < a.n_units; u += blockDim.x)
+      dec_at<DecUnit>(t.units)[u] = dec_unit(a.units[u]);
+  __syncthreads();
+  int* flag = dec_at<int>(t.flag);
   // step end times: CTA 0 stamps each step when the grid barrier after it
   // releases (every CTA has finished it); every CTA stamps the last step's end
   const bool stamp = a.times != nullptr && threadIdx.x == 0;
   if (stamp && blockIdx.x == 0 && a.n_times > 0) a.times[0] = global_ns();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int h = d.h;
   const unsigned G = gridDim.x;
   // phase cycles of thread 0 (shared-memory accumulators): [0] front scan,
   // [1] slot fill, [2] gather + network, [3] per-pixel coding, [4] grid
   // barrier, [5] tiles
-  long long* pc = PROF && a.prof != nullptr ? t.pc : nullptr;
+  long long* pc = PROF && a.prof != nullptr ? dec_at<long long>(t.pc) : nullptr;
   Ticker<PROF> tick(pc);
-  // slots of the tile of n pixels starting at front position base of step
-  // (by the first nt threads)
-  auto fill_slots = [&](int step, long long base, int n, int nt) {
-    for (int s = threadIdx.x; s < n; s += nt) {
-      const int q = (int)(base + s);
-      int lo2 = 0, hi2 = a.n_units - 1;  // last u with pre[u] <= q
-      while (lo2 < hi2) {
-        int mid = (lo2 + hi2 + 1) >> 1;
-        if (t.pre[mid] <= q) lo2 = mid; else hi2 = mid - 1;
-      }
-      const Unit U = a.units[lo2];
-      const Front fr = unit_front(U, step, h, a.sched);
-      DecSlot ps;
-      ps.i = fr.i_lo + (q - t.pre[lo2]);
-      ps.j = front_col(U, step, ps.i, h, a.sched);
-      ps.px = U.img + ((long long)(U.y0 + ps.i) * U.img_W + (U.x0 + ps.j)) * 3;
-      ps.Wu = U.Wu;
-      ps.row_bytes = 3 * U.img_W;
-      ps.stream = U.stream_base + (a.layout == 1 ? ps.i : 0);
-      const bool last = ps.j == U.Wu - 1 && (a.layout == 1 || ps.i == U.Hu - 1);
-      ps.unit = lo2 | (last ? (int)0x80000000 : 0);
-      if constexpr (SHEAR)  // ring bytes of the pixel's sheared column j + (h+1) i
-        t.rofs[s] = kRingRowBytes * (U.ring_row + ps.i) + 3 * ((ps.j + (h + 1) * ps.i) & 15);
-      t.slots[s] = ps;
-    }
-  };
-  // Sheared tile of at most nmax pixels from front position base: the
-  // pixels' slots, their output rows prow (pixel s of the tile's k-th unit
-  // piece at s + h k: each piece is preceded by h halo window rows), the
-  // window rows' (unit, unit row), and t.flag[1..3] = the tile's pixels,
-  // output rows and window rows (the output rows stay below `rows`).
-  auto fill_slots_shear = [&](int step, long long base, int nmax, int nt) {
-    fill_slots(step, base, nmax, nt);
-    part_sync(nt);
-    if ((int)threadIdx.x < rows) {  // warps 0 .. rows/32 - 1
-      const int s = threadIdx.x, w = s >> 5, l = s & 31;
-      const bool valid = s < nmax;
-      const int u = valid ? t.slots[s].unit & 0x7FFFFFFF : -1;
-      const bool start = valid && (s == 0 || u != (t.slots[s - 1].unit & 0x7FFFFFFF));
-      const unsigned bal = __ballot_sync(0xffffffffu, start);
-      if (l == 0) t.sh[w] = __popc(bal);
-      asm volatile("bar.sync 2, %0;" ::"r"(rows) : "memory");
-      int before = 0;
-      for (int k = 0; k < w; k++) before += (int)t.sh[k];
-      const int seg = before + __popc(bal & (0xffffffffu >> (31 - l))) - 1;
-      const int pr = s + h * seg;
-      const bool fits = valid && pr < rows;
-      // the tile's last pixel: the next one is missing or would not fit
-      const bool valid1 = s + 1 < nmax;
-      const int pr1 =
-          s + 1 + h * (seg + ((valid1 && (t.slots[s + 1].unit & 0x7FFFFFFF) != u) ? 1 : 0));
-      t.prow[s] = pr;
-      if (fits) {
-        const int i = t.slots[s].i;
-        t.wrow[pr + h] = make_int2(u, i);
-        if (start)
-          for (int k = 1; k <= h; k++)
-            t.wrow[pr + h - k] = make_int2(i - k >= 0 ? u : -1, i - k);
-        if (!valid1 || pr1 >= rows) {
-          t.flag[1] = s + 1;
-          t.flag[2] = pr + 1;
-          t.flag[3] = pr + 1 + h;
-        }
-      }
-    }
-  };
   // The schedule of step t + 1 (front sizes, this CTA's share, its first
   // tile's slots) needs no decoded data, so it is computed between arriving
   // at the grid barrier after step t and waiting for the others: the last
   // warp arrives (its release waits for the CTA's writes of step t to
   // reach GPU scope) while the other warps compute the schedule.
-  const int NS = (int)blockDim.x - 32;
-  int F = front_scan(a.units, a.n_units, 0, h, a.sched, t.pre, t.sh, (int)blockDim.x);
+  constexpr int NS = NT - 32;
+  sched_front(0, NT);
   tick(0);
-  long long lo = (long long)F * blockIdx.x / G, hi = (long long)F * (blockIdx.x + 1) / G;
-  if (lo < hi) {
-    const int n = (int)min((long long)rows, hi - lo);
-    if constexpr (SHEAR) fill_slots_shear(0, lo, n, (int)blockDim.x);
-    else fill_slots(0, lo, n, (int)blockDim.x);
-  }
+  int lo = flag[6], hi = flag[7];  // the CTA's share of the step's pixels
+  if (lo < hi) sched_slots<SHEAR>(0, lo, min(rows, hi - lo), NT);
   __syncthreads();
   tick(1);
   for (int step = 0; step < a.T; step++) {
-    for (long long base = lo; base < hi;) {
-      int n = (int)min((long long)rows, hi - base);
+    for (int base = lo; base < hi;) {
+      int n = min(rows, hi - base);
       if (base != lo) {  // further tiles of a large share
-        if constexpr (SHEAR) fill_slots_shear(step, base, n, (int)blockDim.x);
-        else fill_slots(step, base, n, (int)blockDim.x);
+        sched_slots<SHEAR>(step, base, n, NT);
         __syncthreads();
       }
-      if constexpr (SHEAR) n = t.flag[1];
+      if constexpr (SHEAR) n = flag[1];
       // A tile with at most one pixel per warp is coded by whole warps (lower
       // latency per pixel); otherwise by quads.  Lane l of warp w copies the
       // stream record of the warp's l-th pixel into shared memory ahead of
@@ -420,9 +561,10 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
       const bool wide = n <= NW;
       const int sl = wide ? (lane == 0 ? warp : rows) : (lane < kQuads ? kQuads * warp + lane : rows);
       if (!SAMPLE && sl < n) {
-        const StreamRec* r = a.st + t.slots[sl].stream;
-        cp_async16(t.rec + sl, r);
-        cp_async16(&t.rec[sl].pos, &r->pos);
+        const StreamRec* r = a.st + dec_at<DecSlot>(t.slots)[sl].stream;
+        StreamRec* rec = dec_at<StreamRec>(t.rec) + sl;
+        cp_async16(rec, r);
+        cp_async16(&rec->pos, &r->pos);
       }
       if (PROF && tick.pc) tick.pc[5] += 1;
       tick(1);
@@ -430,16 +572,16 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
       if constexpr (PREC == PREC_BF16) {
         const long long c0 = PROF && tick.pc ? clock64() : 0;
         if constexpr (SHEAR)
-          net_gather_win(a.units, t.wrow, a.ring, d, t.net, step, t.flag[3]);
-        else if (d.shear) net_gather<true>(t.slots, d, t.net, n);
-        else net_gather<false>(t.slots, d, t.net, n);
+          net_gather_win(a.units, a.ring, t.wrow, step, flag[3]);
+        else if (a.m.d.shear) net_gather<true>(t.slots, n);
+        else net_gather<false>(t.slots, n);
         __syncthreads();
         if (PROF && tick.pc) tick.pc[13] += clock64() - c0;
-        net_ok = net_run<PROF>(d, t.net, SHEAR ? t.flag[2] : n, SHEAR, pc);
+        net_ok = net_run<PROF>(a.m.d.C, SHEAR ? flag[2] : n, SHEAR, phase, pc);
       } else {
-        f32_gather<true>(t.slots, n, d, t.f32);
+        f32_gather<true>(dec_at<DecSlot>(t.slots), n, a.m.d, dec_at<float>(0));
         __syncthreads();
-        f32_run(d, t.f32, n);
+        f32_run(a.m.d, dec_at<float>(0), n);
       }
       // an exchange that timed out: record it and release every CTA from
       // the grid barrier (this one leaves its loop at its next wait)
@@ -450,24 +592,25 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
       if (!SAMPLE) {
         cp_async_wait_all();
         if (sl < n) {
-          const unsigned long long w0 = (t.rec[sl].pos + 8ull) & ~3ull, end = t.rec[sl].end;
+          const unsigned long long w0 = (dec_at<StreamRec>(t.rec)[sl].pos + 8ull) & ~3ull,
+                                   end = dec_at<StreamRec>(t.rec)[sl].end;
 #pragma unroll
           for (int q = 0; q < 3; q++) {
             const unsigned long long wa = w0 + 4ull * q;
-            cp_async4(t.win + 4 * sl + q, a.in + (wa < end ? wa : 0ull), wa < end);
+            cp_async4(dec_at<uint32_t>(t.win) + 4 * sl + q, a.in + (wa < end ? wa : 0ull), wa < end);
           }
         }
         __syncwarp();  // the warp's records are visible to all its lanes
       }
       tick(2);
       if (wide) {
-        code_wide<NW, SAMPLE, SHEAR, PROF>(a, t, n, pc);
+        code_wide<NW, SAMPLE, SHEAR, PROF>(n, pc);
       } else {
-        switch ((d.K + 3) / 4) {
-          case 1: code_quads<1, NW, SAMPLE, SHEAR, PROF>(a, t, n, pc); break;
-          case 2: code_quads<2, NW, SAMPLE, SHEAR, PROF>(a, t, n, pc); break;
-          case 3: code_quads<3, NW, SAMPLE, SHEAR, PROF>(a, t, n, pc); break;
-          default: code_quads<4, NW, SAMPLE, SHEAR, PROF>(a, t, n, pc); break;
+        switch ((a.m.d.K + 3) / 4) {
+          case 1: code_quads<1, NW, SAMPLE, SHEAR, PROF>(n, pc); break;
+          case 2: code_quads<2, NW, SAMPLE, SHEAR, PROF>(n, pc); break;
+          case 3: code_quads<3, NW, SAMPLE, SHEAR, PROF>(n, pc); break;
+          default: code_quads<4, NW, SAMPLE, SHEAR, PROF>(n, pc); break;
         }
       }
       __syncthreads();
@@ -479,27 +622,20 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
     if ((int)threadIdx.x >= NS) {
       if (G > 1 && (int)threadIdx.x == NS) grid_arrive(a.bar);
     } else {
-      F = front_scan(a.units, a.n_units, step + 1, h, a.sched, t.pre, t.sh, NS);
+      sched_front(step + 1, NS);
       tick(0);
-      lo = (long long)F * blockIdx.x / G;
-      hi = (long long)F * (blockIdx.x + 1) / G;
-      if (lo < hi) {
-        const int n = (int)min((long long)rows, hi - lo);
-        if constexpr (SHEAR) fill_slots_shear(step + 1, lo, n, NS);
-        else fill_slots(step + 1, lo, n, NS);
-      }
+      lo = flag[6];
+      hi = flag[7];
+      if (lo < hi) sched_slots<SHEAR>(step + 1, lo, min(rows, hi - lo), NS);
       tick(1);
     }
     if (G > 1) {
-      if (!grid_wait(a.bar, G, target, a.status, t.flag, a.spin_limit)) break;
+      if (!grid_wait(a.bar, G, target, a.status, flag, a.spin_limit)) break;
     } else {
       __syncthreads();
     }
-    if ((int)threadIdx.x >= NS) {
-      F = t.pre[a.n_units];
-      lo = (long long)F * blockIdx.x / G;
-      hi = (long long)F * (blockIdx.x + 1) / G;
-    }
+    lo = flag[6];
+    hi = flag[7];
     tick(4);
     if (stamp && blockIdx.x == 0 && step + 1 < a.n_times) a.times[step + 1] = global_ns();
   }

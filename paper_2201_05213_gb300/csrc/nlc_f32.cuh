@@ -110,7 +110,7 @@ __device__ __forceinline__ void f32_dot(const float* in, int ldm, int Kd, const 
 // writes of X must be visible (a CTA barrier); so is P on return.  MG: number
 // of pixel groups (a power of two).
 template <int PX, int NB>
-__device__ __noinline__ void f32_layers(const Dims& d, float* sm, int n, int MG) {
+__device__ __noinline__ void f32_layers(Dims d, float* sm, int n, int MG) {
   const F32Plan pl = f32_plan(d);
   const int C = d.C, NOp = d.NOp, ldm = f32_ldm(n);
   const int mg = threadIdx.x & (MG - 1), ng = threadIdx.x / MG;
@@ -187,7 +187,7 @@ __device__ __forceinline__ void f32_run(const Dims& d, float* sm, int n) {
 // Context tile of the slots (Slot: px, i, j, Wu, row_bytes as in DecSlot),
 // feature-major.  kCoherent: the image is being decoded (loads through L2).
 template <bool kCoherent, class Slot>
-__device__ __forceinline__ void f32_gather(const Slot* slots, int n, const Dims& d, float* sm) {
+__device__ __forceinline__ void f32_gather(const Slot* slots, int n, const Dims d, float* sm) {
   float* X = sm + f32_plan(d).u;
   const int h = d.h, ldm = f32_ldm(n), ntap = 2 * h * (h + 1), np = ldm - 4;
   const int lg = 31 - __clz(np);

@@ -69,48 +69,45 @@ __host__ __device__ inline NetPlan net_plan(const Dims& d, int rows, bool win) {
   return p;
 }
 
+// The decoder's dynamic shared memory: first a record of kSharedHead bytes (its
+// beginning is the NetSmem), then the regions of the plans.  Its functions
+// address it through this symbol and offsets, never through pointers kept in
+// memory: those would be generic addresses, and their loads slower.
+extern __shared__ __align__(128) unsigned char dec_smem[];
+constexpr int kSharedHead = 640;
+template <class T>
+__device__ __forceinline__ T* dec_at(int off) {
+  return reinterpret_cast<T*>(dec_smem + kSharedHead + off);
+}
+
 struct NetSmem {
-  unsigned char* base;
-  uint16_t* X;
-  float* P;
-  float* bias;
-  uint64_t* mbar;
+  Dims d;
+  NetPlan pl;
   int rows;
-  uint32_t phase;  // bit l: parity of the warp's mbarrier when m-tiles have 8 >> l warps
   unsigned limit;  // polls of an exchange before a timeout is recorded
 };
-
-__device__ __forceinline__ NetSmem net_carve(const Dims& d, unsigned char* smem, int rows,
-                                             bool win) {
-  const NetPlan p = net_plan(d, rows, win);
-  NetSmem t;
-  t.base = smem;
-  t.X = reinterpret_cast<uint16_t*>(smem + p.x);
-  t.P = reinterpret_cast<float*>(smem + p.x);
-  t.bias = reinterpret_cast<float*>(smem + p.bias);
-  t.mbar = reinterpret_cast<uint64_t*>(smem + p.mbar);
-  t.rows = rows;
-  t.phase = 0;
-  t.limit = kMbarSpin;
-  return t;
+__device__ __forceinline__ const NetSmem& net_smem() {
+  return *reinterpret_cast<const NetSmem*>(dec_smem);
 }
 
 // One thread; a CTA barrier must follow.
-__device__ __forceinline__ void net_setup(NetSmem& t) {
+__device__ __forceinline__ void net_setup(const NetPlan& pl) {
   for (int i = 0; i < kNetBars; i++) {
     const uint32_t count = i < 2 ? 8u : i < 6 ? 4u : 2u;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(t.mbar + i)), "r"(count)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(
+                     smem_u32(dec_at<uint64_t>(pl.mbar) + i)),
+                 "r"(count)
                  : "memory");
   }
 }
 
-__device__ __forceinline__ void net_load_weights(const Dims& d, const WeightView& w, NetSmem& t) {
+__device__ __forceinline__ void net_load_weights(const Dims& d, const WeightView& w, int bias) {
   const int nh = w.umma_halves;  // multiple of 64 (core matrices)
   const uint4* src = reinterpret_cast<const uint4*>(w.umma);
-  uint4* dst = reinterpret_cast<uint4*>(t.base);
+  uint4* dst = dec_at<uint4>(0);
   for (int i = threadIdx.x; i < nh / 8; i += blockDim.x) dst[i] = src[i];
   const int nb = (int)bias_floats(d);
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) t.bias[i] = w.bias[i];
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) dec_at<float>(bias)[i] = w.bias[i];
 }
 
 // ldmatrix / mma.sync.  Volatile without a memory clobber: they keep their
@@ -133,6 +130,29 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
       "{%8,%9}, {%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Two FP32 operations in one instruction, each rounded as its scalar form.
+__device__ __forceinline__ void add2(float& a, float& b, float x, float y) {
+  asm("{\n.reg .b64 p, q;\nmov.b64 p, {%0, %1};\nmov.b64 q, {%2, %3};\n"
+      "add.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
+      : "+f"(a), "+f"(b)
+      : "f"(x), "f"(y));
+}
+__device__ __forceinline__ void mul2(float& a, float& b, float x) {
+  asm("{\n.reg .b64 p, q;\nmov.b64 p, {%0, %1};\nmov.b64 q, {%2, %2};\n"
+      "mul.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
+      : "+f"(a), "+f"(b)
+      : "f"(x));
+}
+// ELU of two values (elu_tc's steps) as a BF16 pair.
+__device__ __forceinline__ uint32_t elu_pair(float x, float y) {
+  float a = x, b = y;
+  mul2(a, b, 1.4426950408889634f);
+  a = ex2_approx(a);
+  b = ex2_approx(b);
+  add2(a, b, -1.f, -1.f);
+  return pack_bf16(x > 0.f ? x : a, y > 0.f ? y : b);
 }
 
 // B fragments of KS K steps of one 8-column tile (addr: the lane's row in the
@@ -174,32 +194,33 @@ __device__ __forceinline__ bool net_exchange(uint64_t* mb, int mt, int threads, 
 // that a layer is straight-line code: its B fragments are loaded before the
 // exchange that precedes it, its A fragments right after.
 template <int NT8, int LEVEL, bool PROF>
-__device__ __noinline__ bool net_layers(const Dims& d, NetSmem& t, int n, bool win,
-                                        long long* pc) {
+__device__ __noinline__ uint32_t net_layers(int n, bool win, uint32_t phase, long long* pc) {
   constexpr int NS = 8 >> LEVEL, KS = NT8 / 2, TP = (NT8 + NS - 1) / NS;
   constexpr int HG = LEVEL == 0 ? 1 : LEVEL == 1 ? 2 : 4;  // head tiles computed together
   constexpr uint32_t kWBytes = 128u * NT8 * NT8;  // bytes of a hidden layer's weights
-  const NetPlan pl = net_plan(d, t.rows, win);
+  const NetSmem& t = net_smem();
+  const Dims& d = t.d;
+  const NetPlan& pl = t.pl;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mt = warp / NS, ns = warp % NS;
   const bool live = 16 * mt < n;
   const int g = lane >> 2, q = lane & 3;
-  const uint32_t sb = smem_u32(t.base);
+  const uint32_t sb = smem_u32(dec_smem) + (uint32_t)kSharedHead;
   const uint32_t cs = (uint32_t)t.rows * 16u;  // bytes of a chunk
   // ldmatrix rows: lanes 0-7 rows 0-7, 8-15 rows 8-15 of the even chunk, then the odd chunk
   const uint32_t arow = sb + (uint32_t)(16 * mt + (lane & 15)) * 16u + (uint32_t)(lane >> 4) * cs;
   const uint32_t brow = sb + (uint32_t)(lane & 7) * 16u;
-  uint64_t* mb = t.mbar + (LEVEL == 0 ? 0 : LEVEL == 1 ? 2 : 6) + mt;
+  uint64_t* mb = dec_at<uint64_t>(pl.mbar) + (LEVEL == 0 ? 0 : LEVEL == 1 ? 2 : 6) + mt;
   const bool pr = PROF && pc != nullptr && threadIdx.x == 0;
   long long ck = pr ? clock64() : 0;
-  uint32_t parity = (t.phase >> LEVEL) & 1u;
+  uint32_t parity = (phase >> LEVEL) & 1u;
   const unsigned limit = t.limit;
   const int n_hidden = 1 + 2 * d.R, nht = (d.NO + 7) / 8;
   const uint32_t x = arow + (uint32_t)pl.x, h0 = arow + (uint32_t)pl.h0, h1 = arow + (uint32_t)pl.h1;
-  const float* bias = t.bias + 2 * q;
+  const float* bias = dec_at<float>(pl.bias) + 2 * q;
   // the lane's columns 2q, 2q + 1 of rows g, g + 8 of the m-tile
-  unsigned char* o0 = t.base + pl.h0 + (16 * mt + g) * 16 + q * 4;
-  unsigned char* o1 = t.base + pl.h1 + (16 * mt + g) * 16 + q * 4;
+  unsigned char* o0 = dec_at<unsigned char>(pl.h0) + (16 * mt + g) * 16 + q * 4;
+  unsigned char* o1 = dec_at<unsigned char>(pl.h1) + (16 * mt + g) * 16 + q * 4;
   bool ok = true;
   if (live) {
     auto on = [&](int i) { return NT8 % NS == 0 || ns + NS * i < NT8; };
@@ -260,17 +281,18 @@ __device__ __noinline__ bool net_layers(const Dims& d, NetSmem& t, int n, bool w
       for (int i = 0; i < TP; i++) {
         const int j = tile(i);
         const float2 bb = *reinterpret_cast<const float2*>(b + 8 * j);
-        float u[4];
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-          float v = __fadd_rn(acc[i][e], (e & 1) ? bb.y : bb.x);
-          if (M == 1) v = __fadd_rn(res[i][e], v);
-          if (M != 2) res[i][e] = v;
-          u[e] = elu_tc(v);
+        add2(acc[i][0], acc[i][1], bb.x, bb.y);
+        add2(acc[i][2], acc[i][3], bb.x, bb.y);
+        if (M == 1) {
+          add2(acc[i][0], acc[i][1], res[i][0], res[i][1]);
+          add2(acc[i][2], acc[i][3], res[i][2], res[i][3]);
         }
+        if (M != 2)
+#pragma unroll
+          for (int e = 0; e < 4; e++) res[i][e] = acc[i][e];
         if (on(i)) {
-          *reinterpret_cast<uint32_t*>(o + j * cs) = pack_bf16(u[0], u[1]);
-          *reinterpret_cast<uint32_t*>(o + j * cs + 128) = pack_bf16(u[2], u[3]);
+          *reinterpret_cast<uint32_t*>(o + j * cs) = elu_pair(acc[i][0], acc[i][1]);
+          *reinterpret_cast<uint32_t*>(o + j * cs + 128) = elu_pair(acc[i][2], acc[i][3]);
         }
       }
     };
@@ -311,7 +333,7 @@ __device__ __noinline__ bool net_layers(const Dims& d, NetSmem& t, int n, bool w
       wl += 2 * kWBytes;
       bias += 16 * NT8;
     }
-    t.phase = (t.phase & ~(1u << LEVEL)) | (parity << LEVEL);
+    phase = (phase & ~(1u << LEVEL)) | (parity << LEVEL);
   }
   // The head on all warps: every m-tile gets 16 / m-tiles of them.  The CTA
   // barrier is the last exchange and keeps P off the tiles it aliases.
@@ -328,8 +350,8 @@ __device__ __noinline__ bool net_layers(const Dims& d, NetSmem& t, int n, bool w
     const uint32_t h = sb + (uint32_t)pl.h0 + (uint32_t)(16 * hm + (lane & 15)) * 16u +
                        (uint32_t)(lane >> 4) * cs;
     const int ldp = net_ldp(d);
-    const float* bh = t.bias + 8 * NT8 * n_hidden + 2 * q;
-    float* o = t.P + (size_t)(16 * hm + g) * ldp + 2 * q;
+    const float* bh = dec_at<float>(pl.bias) + 8 * NT8 * n_hidden + 2 * q;
+    float* o = dec_at<float>(pl.x) + (16 * hm + g) * ldp + 2 * q;
     uint32_t a[KS][4];
 #pragma unroll
     for (int s = 0; s < KS; s++)
@@ -364,30 +386,33 @@ __device__ __noinline__ bool net_layers(const Dims& d, NetSmem& t, int n, bool w
   }
   __syncthreads();
   if (pr) pc[15] += clock64() - ck;
-  return all_ok != 0;
+  return phase | (all_ok ? 0x80000000u : 0u);
 }
 
 // The whole network on the n pixels (n >= 1) of the context tile: P[m][ldp]
 // = head outputs, visible to the CTA on return.  win: X is the sheared
 // decoder's window tile (rows 16 bytes apart, (rows + 8) per chunk).  Returns
-// false (in every thread) if an exchange timed out.  PROF: thread 0 adds its
-// cycles of the hidden layers to pc[14] and those of the head to pc[15].
+// false (in every thread) if an exchange timed out.  phase: the caller's record
+// of the warp's mbarrier parities (bit l: m-tiles of 8 >> l warps), 0 at
+// first.  PROF: thread 0 adds its cycles of the hidden layers to pc[14] and
+// those of the head to pc[15].
 template <int NT8, bool PROF>
-__device__ __forceinline__ bool net_levels(const Dims& d, NetSmem& t, int n, bool win,
-                                           long long* pc) {
-  if (n <= 32) return net_layers<NT8, 0, PROF>(d, t, n, win, pc);
-  if (n <= 64) return net_layers<NT8, 1, PROF>(d, t, n, win, pc);
-  return net_layers<NT8, 2, PROF>(d, t, n, win, pc);
+__device__ __forceinline__ uint32_t net_levels(int n, bool win, uint32_t phase, long long* pc) {
+  if (n <= 32) return net_layers<NT8, 0, PROF>(n, win, phase, pc);
+  if (n <= 64) return net_layers<NT8, 1, PROF>(n, win, phase, pc);
+  return net_layers<NT8, 2, PROF>(n, win, phase, pc);
 }
 template <bool PROF>
-__device__ __forceinline__ bool net_run(const Dims& d, NetSmem& t, int n, bool win,
-                                        long long* pc) {
-  switch (d.C / 8) {
-    case 2: return net_levels<2, PROF>(d, t, n, win, pc);
-    case 4: return net_levels<4, PROF>(d, t, n, win, pc);
-    case 6: return net_levels<6, PROF>(d, t, n, win, pc);
-    default: return net_levels<8, PROF>(d, t, n, win, pc);
+__device__ __forceinline__ bool net_run(int C, int n, bool win, uint32_t& phase, long long* pc) {
+  uint32_t r;
+  switch (C / 8) {
+    case 2: r = net_levels<2, PROF>(n, win, phase, pc); break;
+    case 4: r = net_levels<4, PROF>(n, win, phase, pc); break;
+    case 6: r = net_levels<6, PROF>(n, win, phase, pc); break;
+    default: r = net_levels<8, PROF>(n, win, phase, pc); break;
   }
+  phase = r & 0x7FFFFFFFu;
+  return (r >> 31) != 0;
 }
 
 // --- context tiles ------------------------------------------------------------
@@ -496,17 +521,20 @@ __device__ __forceinline__ void gather_row_shear(const Slot& s, int dd, int h, i
 
 // The decoder's tile, from its slots: a warp covers 8 pixels x 4 rows.
 template <bool SHEAR>
-__device__ __noinline__ void net_gather(const DecSlot* slots, const Dims& d, NetSmem& t, int n) {
+__device__ __noinline__ void net_gather(int slots, int n) {
+  const NetSmem& t = net_smem();
+  const Dims d = t.d;
+  uint16_t* X = dec_at<uint16_t>(t.pl.x);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r = lane >> 3, cs = 8 * t.rows;
   for (int mb = 8 * warp; mb < n; mb += 8 * (int)(blockDim.x >> 5)) {
     const int m = mb + (lane & 7);
     if (r > d.h || m >= n) continue;
-    const DecSlot s = slots[m];
+    const DecSlot s = dec_at<DecSlot>(slots)[m];
     if (SHEAR)
-      gather_row_shear<true>(s, r, d.h, d.Ws, d.Fsp, t.X + (size_t)r * (d.Fsp / 8) * cs + 8 * m, cs);
+      gather_row_shear<true>(s, r, d.h, d.Ws, d.Fsp, X + r * (d.Fsp / 8) * cs + 8 * m, cs);
     else
-      gather_row<true>(s, r, d.h, d.F, d.Fp, t.X + 8 * m, cs);
+      gather_row<true>(s, r, d.h, d.F, d.Fp, X + 8 * m, cs);
   }
 }
 
@@ -516,15 +544,16 @@ __device__ __noinline__ void net_gather(const DecSlot* slots, const Dims& d, Net
 // started dd rows further.  wrow[rho] = (unit, unit row) of window row rho
 // (unit -1: a zero row); the decoded pixels come from the units' sheared
 // rings (unit u's row r at ring + 96 (u.ring_row + r)).
-static __device__ __noinline__ void net_gather_win(const Unit* units, const int2* wrow,
-                                                   const uint8_t* ring, const Dims& d, NetSmem& t,
-                                                   int step, int n_rows) {
-  const int h = d.h, Ws = d.Ws, nch = d.Fsp / 8, wr8 = 8 * (t.rows + 8);
+static __device__ __noinline__ void net_gather_win(const Unit* units, const uint8_t* ring,
+                                                   int wrow_off, int step, int n_rows) {
+  const NetSmem& t = net_smem();
+  const int2* wrow = dec_at<int2>(wrow_off);
+  const int h = t.d.h, Ws = t.d.Ws, nch = t.d.Fsp / 8, wr8 = 8 * (t.rows + 8);
   // window columns step - Ws .. step - 1: ring bytes from 3 ((step - Ws) mod 16);
   // feature k of a window row is byte k of that range
   const int c0 = step - Ws;
   const int b0 = 3 * (c0 & 15);
-  uint16_t* X = t.X;
+  uint16_t* X = dec_at<uint16_t>(t.pl.x);
   // one item per (window row, 8-feature chunk); rows past n_rows feed only
   // output rows that hold no pixel and are left as they are
   for (int it = threadIdx.x; it < n_rows * nch; it += blockDim.x) {

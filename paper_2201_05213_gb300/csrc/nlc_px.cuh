@@ -78,29 +78,6 @@ __device__ __forceinline__ int px_slots(const Unit* __restrict__ units, int n_un
   return hint;
 }
 
-// Two FP32 operations in one instruction, each rounded as its scalar form.
-__device__ __forceinline__ void add2(float& a, float& b, float x, float y) {
-  asm("{\n.reg .b64 p, q;\nmov.b64 p, {%0, %1};\nmov.b64 q, {%2, %3};\n"
-      "add.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
-      : "+f"(a), "+f"(b)
-      : "f"(x), "f"(y));
-}
-__device__ __forceinline__ void mul2(float& a, float& b, float x) {
-  asm("{\n.reg .b64 p, q;\nmov.b64 p, {%0, %1};\nmov.b64 q, {%2, %2};\n"
-      "mul.rn.f32x2 p, p, q;\nmov.b64 {%0, %1}, p;\n}\n"
-      : "+f"(a), "+f"(b)
-      : "f"(x));
-}
-// ELU of two values (elu_tc's steps) as a BF16 pair.
-__device__ __forceinline__ uint32_t elu_pair(float x, float y) {
-  float a = x, b = y;
-  mul2(a, b, 1.4426950408889634f);
-  a = ex2_approx(a);
-  b = ex2_approx(b);
-  add2(a, b, -1.f, -1.f);
-  return pack_bf16(x > 0.f ? x : a, y > 0.f ? y : b);
-}
-
 // Network up to the head's input: fragments a[s] of ELU(a_R) for the warp's 16
 // pixels, from the context tile at x (chunks of 256 bytes).
 template <int NT8>

@@ -71,31 +71,6 @@ __device__ __forceinline__ long long block_excl_scan(long long v, long long* sh,
   return block_excl_scan(v, sh, total, (int)blockDim.x);
 }
 
-// Fronts of all units at global step t: pre[u] = exclusive prefix of the
-// front sizes, pre[n_units] = total.  Requires n_units + 1 ints of smem.
-// Computed by (and returned to) the first nt threads of the CTA.
-__device__ __forceinline__ int front_scan(const Unit* __restrict__ units, int n_units, int t,
-                                          int h, int sched, int* pre, long long* sh, int nt) {
-  const int per = (n_units + nt - 1) / nt;
-  const int u0 = threadIdx.x * per, u1 = min(u0 + per, n_units);
-  long long sum = 0;
-  for (int u = u0; u < u1; u++) {
-    int c = unit_front(units[u], t, h, sched).n;
-    pre[u] = c;
-    sum += c;
-  }
-  long long total;
-  long long run = block_excl_scan(sum, sh, &total, nt);
-  for (int u = u0; u < u1; u++) {
-    int c = pre[u];
-    pre[u] = (int)run;
-    run += c;
-  }
-  if (threadIdx.x == 0) pre[n_units] = (int)total;
-  part_sync(nt);
-  return (int)total;
-}
-
 // ---------------------------------------------------------------------
 // rANS: warp-level decoder of one stream position and the per-stream
 // encoder (byte-wise renormalisation, state in [2^23, 2^31)).
