@@ -16,7 +16,7 @@
 // The weight-gradient chains use M = 128 rows of which the first n_out are
 // the layer's outputs (the others read the neighbouring core matrices and
 // are discarded).  Each layer's weight and bias gradients are added to the
-// CTA's own FP32 slot in global memory after its chain completes (every
+// CTA's own FP32 slot in global memory behind the next layer's chains (every
 // element by one thread, tiles in a fixed order), and a second kernel sums
 // the slots in a fixed order: the result is deterministic.
 //
@@ -24,40 +24,50 @@
 // folded into W0, so its gradient is scaled by 1/255 on the way out), then
 // u = ELU(a) and v = ELU(z) in BF16; ELU'(t) = 1 for t > 0 and ELU(t) + 1
 // otherwise, taken from the stored BF16 activation.  The residual stream and
-// its gradient stay in FP32 registers.  The mixture likelihood and its
+// its gradient stay in FP32 in tensor memory.  The mixture likelihood and its
 // gradient with respect to the 10K network outputs are FP32; the outputs are
-// read straight from tensor memory (two threads per pixel, each holding
-// every other mixture component) and the gradient is stored in BF16 as the
-// A operand of the head's adjoint.  256 threads per CTA: each thread owns a
-// pixel row and half of its columns, within the register budget.
+// read straight from tensor memory (four threads per pixel, each holding
+// every fourth mixture component) and the gradient is stored in BF16 as the
+// A operand of the head's adjoint.  512 threads per CTA: each thread owns a
+// pixel row and a quarter of its columns.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "nlc_common.cuh"
+#include "nlc_mma.cuh"
 #include "nlc_model.cuh"
 #include "nlc_tc.cuh"
 #include "nlc_train.cuh"
 
 namespace nlc {
 
-constexpr int kTT = 256;                  // threads (8 warps)
+constexpr int kTT = 512;                  // threads (16 warps)
 constexpr int kTTM = 128;                 // pixels per tile (the MMA's M)
 constexpr int kParts = kTT / kTTM;        // threads per pixel row (column parts)
 constexpr uint32_t kTTCols = 512;         // tensor-memory columns
 constexpr uint32_t kColAcc = 0;           // forward / adjoint accumulator (N <= 160)
-constexpr uint32_t kColDW = 256;          // weight-gradient accumulator (N <= Fp <= 80)
-constexpr uint32_t kColDB = 384;          // bias-gradient accumulator (N = 16)
 constexpr uint32_t kColRes = 400;         // residual stream / its gradient (FP32, C <= 64)
 constexpr int kCompPerThread = (kMaxK + kParts - 1) / kParts;
-constexpr int kChunks = (kMaxC / 8 + kParts - 1) / kParts;  // 8-column chunks per thread
+// Weight- and bias-gradient accumulators (N <= Fp <= 80 and N = 16): two of
+// each, so that a layer's are added to the slot while the next layer's chains
+// run.
+__device__ __forceinline__ constexpr uint32_t col_dw(int b) { return b ? 160u : 256u; }
+__device__ __forceinline__ constexpr uint32_t col_db(int b) { return b ? 240u : 384u; }
 constexpr int kLbStride = kMaxK + 1;  // per-row table of l_k (odd: rows on different banks)
+
+// One pixel of the tile: its position in its image; i = -1 for pixels past the
+// batch (their context is then zero).
+struct TTSlot {
+  int i, j;
+};
 
 // Byte offsets of the shared-memory regions.  Residual block r's tiles are
 // at w1 + r * wstride (W1) and w1 + r * wstride + wstride / 2 (W2): plain
 // arithmetic, so that no offset table has to live in local memory.
 struct TTPlan {
   int w0, w1, wstride, wh;  // BF16 weight tiles (the decoder's layout)
-  int bias, ones, u, gx, g2, xe, red, slots, taps, mbar, tslot, end;
+  int bias, ones, u, gx, g2, x, xe, red, slots, mbar, tslot, end;
+  bool keep_x;  // X stays in a region of its own from the forward to its weight gradient
   bool fits;
 };
 
@@ -80,31 +90,38 @@ __host__ __device__ inline TTPlan tt_plan(const Dims& d) {
   o += 512;
   p.u = o;  // 2R+1 activation tiles [128][C]
   o += (2 * d.R + 1) * tile_bytes(d.C);
-  // gradient region: X during the forward, then dP [128][NOp] with the
+  // gradient region: (X during the forward,) then dP [128][NOp] with the
   // likelihood's per-row table [128][17], then G and G2 [128][C]
   p.gx = o;
   p.g2 = o + tile_bytes(d.C);
-  const int dp = tile_bytes(d.NOp);
+  const int dp = tile_bytes(d.NOp), xb = tile_bytes(d.Fp);
   p.red = o + dp;
   int need = dp + kTTM * kLbStride * 4;
   if (need < 2 * tile_bytes(d.C)) need = 2 * tile_bytes(d.C);
-  if (need < tile_bytes(d.Fp)) need = tile_bytes(d.Fp);
-  // X for the first layer's weight gradient, gathered again after the
-  // adjoint: into the activation tiles when they are large enough
-  if ((2 * d.R + 1) * tile_bytes(d.C) >= tile_bytes(d.Fp)) {
-    p.xe = p.u;
+  // the weight-gradient chains read up to (128 - n_out)/8 core matrices past a
+  // gradient tile's end (discarded rows): keep them inside the block
+  const int tail = 1024 + kTTM * (int)sizeof(TTSlot) + 16 + 128;
+  p.keep_x = o + need + xb + tail <= 227 * 1024;
+  if (p.keep_x) {
+    p.x = p.xe = o + need;
+    o += need + xb;
   } else {
-    p.xe = o + tile_bytes(d.C);
-    if (need < tile_bytes(d.C) + tile_bytes(d.Fp)) need = tile_bytes(d.C) + tile_bytes(d.Fp);
+    // X shares the gradient region in the forward and is gathered again for
+    // its weight gradient, into the activation tiles when they are large enough
+    if (need < xb) need = xb;
+    p.x = o;
+    if ((2 * d.R + 1) * tile_bytes(d.C) >= xb) {
+      p.xe = p.u;
+    } else {
+      p.xe = o + tile_bytes(d.C);
+      if (need < tile_bytes(d.C) + xb) need = tile_bytes(d.C) + xb;
+    }
+    o += need;
   }
-  // the weight-gradient chains read up to (128 - n_out)/8 core matrices
-  // past a gradient tile's end (discarded rows): keep them inside the block
-  o += need + 1024;
+  o += 1024;
   o = align_up(o, 16);
-  p.slots = o;  // (image, i, j, valid) per pixel
-  o += kTTM * 16;
-  p.taps = o;  // (dy, dx) of the context taps (Eq. 3), 2h(h+1) <= 24
-  o += 24 * 8;
+  p.slots = o;
+  o += kTTM * (int)sizeof(TTSlot);
   p.mbar = o;
   o += 8;
   p.tslot = o;
@@ -181,98 +198,85 @@ __device__ __forceinline__ float elu_t(float x) {
 // ELU'(t) from the stored activation u = ELU(t)
 __device__ __forceinline__ float elu_d_from_act(float u) { return u > 0.f ? 1.f : u + 1.f; }
 
-// X tile [128][Fp] (K-major): feature 3p + c of pixel m = 2v - 255 of channel
-// c of context tap p (Eq. 3), 0 outside the image and for F <= k < Fp and for
-// rows past the batch.  Pixel m's (image, row, column, valid) come from the
-// tile's slot table and tap p's offsets from taps[p], so that no index is
-// divided per feature; thread t handles pixel t mod 128.
-__device__ __noinline__ void tt_gather(const Dims& d, const uint8_t* __restrict__ batch, int H,
-                                       int W, const int4* slots, const int2* taps,
-                                       unsigned char* X) {
-  const int ntap = d.F / 3, Fp = d.Fp;
-  uint16_t* x = reinterpret_cast<uint16_t*>(X);
-  const int m = threadIdx.x & (kTTM - 1);
-  const int4 sl = slots[m];
-  const long long base = ((long long)sl.x * H) * W;
-  for (int p = threadIdx.x / kTTM; 3 * p < Fp; p += kTT / kTTM) {
-    float v[3] = {0.f, 0.f, 0.f};
-    if (sl.w != 0 && p < ntap) {
-      const int2 t = taps[p];
-      const int ii = sl.y + t.x, jj = sl.z + t.y;
-      if (ii >= 0 && ii < H && jj >= 0 && jj < W) {
-        const uint8_t* px = batch + (base + (long long)ii * W + jj) * 3;
-        v[0] = (float)(2 * (int)px[0] - 255);
-        v[1] = (float)(2 * (int)px[1] - 255);
-        v[2] = (float)(2 * (int)px[2] - 255);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; c++)
-      if (3 * p + c < Fp)
-        x[umma_off(m, 3 * p + c, Fp)] = __bfloat16_as_ushort(__float2bfloat16_rn(v[c]));
-  }
+// X tile [128][Fp] (K-major): the pixels' contexts (gather_row), one thread
+// per (pixel, context row).
+__device__ __noinline__ void tt_gather(const Dims& d, const uint8_t* px0, int W,
+                                       const TTSlot* slots, unsigned char* X) {
+  const int m = threadIdx.x & (kTTM - 1), r = threadIdx.x / kTTM;
+  static_assert(kTT / kTTM == kMaxH + 1, "one context row per thread");
+  if (r > d.h) return;
+  struct {
+    const uint8_t* px;
+    int i, j, Wu, row_bytes;
+  } s{px0 + 3 * m, slots[m].i, slots[m].j, W, 3 * W};
+  gather_row<false>(s, r, d.h, d.F, d.Fp,
+                    reinterpret_cast<uint16_t*>(X) + (m >> 3) * (d.Fp >> 3) * 64 + (m & 7) * 8, 64);
+}
+
+__device__ __forceinline__ void red_add2(float* p, float a, float b) {
+  asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b)
+               : "memory");
+}
+__device__ __forceinline__ void red_add1(float* p, float a) {
+  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory");
+}
+
+// 16 rows x 8 FP32 columns of tensor memory, without waiting: lane l gets
+// columns 2 (l % 4), + 1 of rows l / 4 (r[0], r[1]) and l / 4 + 8 (r[2], r[3]).
+__device__ __forceinline__ void tmem_ld16x8_nw(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
 }
 
 // Adds the weight gradient of one layer (D rows o < n_out, columns i < n_in
-// of the weight-gradient accumulator, times `scale`) and its bias gradient
-// (column 0 of the bias accumulator) to the CTA's slot (16-byte aligned rows
-// when n_in and ld are multiples of 4).  All tensor-memory loads, then all
-// global loads, then the stores: one memory round trip per layer.
-constexpr int kFlushChunks = (80 / 8 + kParts - 1) / kParts;  // n_in <= 80
-__device__ __noinline__ void tt_flush(uint32_t tmem, int n_out, int n_in, int ld, float scale,
-                         float* __restrict__ gW, float* __restrict__ gb) {
+// of weight-gradient accumulator `buf`, times `scale`) and its bias gradient
+// (column 0 of the bias accumulator) to the CTA's slot, as reductions: an
+// element is always added to by the same thread, tile after tile, so their
+// order is fixed, and no thread waits for the old value.  Four neighbouring
+// lanes hold 32 consecutive bytes of a row (n_in and ld are even), so that a
+// warp's reduction touches eight whole sectors instead of 32 rows.
+__device__ __noinline__ void tt_flush(uint32_t tmem, int buf, int n_out, int n_in, int ld,
+                                      float scale, float* __restrict__ gW,
+                                      float* __restrict__ gb) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3, part = warp >> 2;
-  const int o = 32 * q + lane;
   if (32 * q >= n_out) return;  // whole warp outside the layer's outputs
   const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
   const int nch = (n_in + 7) / 8;
-  uint32_t r[kFlushChunks][8];
-#pragma unroll
-  for (int i = 0; i < kFlushChunks; i++)
-    if (part + kParts * i < nch) tmem_ld8_nw(tl + kColDW + 8 * (part + kParts * i), r[i]);
-  uint32_t rb[8];
-  if (part == 0) tmem_ld8_nw(tl + kColDB, rb);
-  tmem_wait_ld();
-  if (o >= n_out) return;
-  float* row = gW + (size_t)o * ld;
-  float4 g[kFlushChunks][2];
-#pragma unroll
-  for (int i = 0; i < kFlushChunks; i++) {
-    const int c = part + kParts * i;
-    if (c < nch && 8 * c + 8 <= n_in) {
-      g[i][0] = *reinterpret_cast<const float4*>(row + 8 * c);
-      g[i][1] = *reinterpret_cast<const float4*>(row + 8 * c + 4);
+#pragma unroll 1
+  for (int c = part; c < nch; c += kParts) {
+    uint32_t r0[4], r1[4];
+    tmem_ld16x8_nw(tl + col_dw(buf) + 8 * c, r0);
+    tmem_ld16x8_nw(tl + (16u << 16) + col_dw(buf) + 8 * c, r1);
+    tmem_wait_ld();
+    asm volatile("" : "+r"(r0[0]), "+r"(r0[1]), "+r"(r0[2]), "+r"(r0[3]));
+    asm volatile("" : "+r"(r1[0]), "+r"(r1[1]), "+r"(r1[2]), "+r"(r1[3]));
+    const int col = 8 * c + 2 * (lane & 3), o = 32 * q + (lane >> 2);
+    float* p = gW + (size_t)o * ld + col;
+    if (col < n_in) {
+      auto put = [&](int k, uint32_t x, uint32_t y) {  // row o + 8 k
+        if (o + 8 * k < n_out)
+          red_add2(p + (size_t)(8 * k) * ld, __fmul_rn(__uint_as_float(x), scale),
+                   __fmul_rn(__uint_as_float(y), scale));
+      };
+      put(0, r0[0], r0[1]);
+      put(1, r0[2], r0[3]);
+      put(2, r1[0], r1[1]);
+      put(3, r1[2], r1[3]);
     }
-  }
-  const float gbo = part == 0 ? gb[o] : 0.f;
-#pragma unroll
-  for (int i = 0; i < kFlushChunks; i++) {
-    const int c = part + kParts * i;
-    if (c >= nch) continue;
-    tmem_touch(r[i]);
-    float v[8];
-#pragma unroll
-    for (int e = 0; e < 8; e++) v[e] = __fmul_rn(__uint_as_float(r[i][e]), scale);
-    if (8 * c + 8 <= n_in) {
-      float4 a = g[i][0], b = g[i][1];
-      a.x = __fadd_rn(a.x, v[0]);
-      a.y = __fadd_rn(a.y, v[1]);
-      a.z = __fadd_rn(a.z, v[2]);
-      a.w = __fadd_rn(a.w, v[3]);
-      b.x = __fadd_rn(b.x, v[4]);
-      b.y = __fadd_rn(b.y, v[5]);
-      b.z = __fadd_rn(b.z, v[6]);
-      b.w = __fadd_rn(b.w, v[7]);
-      *reinterpret_cast<float4*>(row + 8 * c) = a;
-      *reinterpret_cast<float4*>(row + 8 * c + 4) = b;
-    } else {  // ragged last chunk
-      for (int e = 0; e < 8 && 8 * c + e < n_in; e++) row[8 * c + e] = __fadd_rn(row[8 * c + e], v[e]);
-    }
+    __syncwarp();
   }
   if (part == 0) {
-    tmem_touch(rb);
-    gb[o] = __fadd_rn(gbo, __uint_as_float(rb[0]));
+    uint32_t rb;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
+                 : "=r"(rb)
+                 : "r"(tl + col_db(buf))
+                 : "memory");
+    tmem_wait_ld();
+    asm volatile("" : "+r"(rb));
+    if (32 * q + lane < n_out) red_add1(gb + 32 * q + lane, __uint_as_float(rb));
   }
 }
 
@@ -393,37 +397,42 @@ __device__ __noinline__ float tt_likelihood(const Dims& d, uint32_t tcol, const 
     __syncthreads();
     const float lse_pi = row_lse();
     __syncthreads();
-    // locations m_c (coupled), log-scales, the channel log-masses, and with
-    // want_d the derivatives of each channel's log-mass with respect to its
-    // location (dlm) and log-scale (dll)
-    auto comp_terms = [&](const float (&pr)[10], float (&co)[3], float (&dlm)[3],
-                          float (&dll)[3], bool want_d) {
-      float lk = 0.f;
+    // Per component: locations m_c (coupled), log-scales, l_k = log pi_k +
+    // sum_c log P_c,k, and the derivatives of each channel's log-mass with
+    // respect to its location (dlm) and log-scale (dll; 0 where it is
+    // clamped); kept in registers until log p is known.
+    float lk_[kCompPerThread], dlm[kCompPerThread][3], dll[kCompPerThread][3];
+#pragma unroll
+    for (int i = 0; i < kCompPerThread; i++) {
+      const int k = part + kParts * i;
+      if (k >= K) continue;
+      float pr[10];
+      load_comp(k, pr);
+      float lk = 0.f, co[3];
 #pragma unroll
       for (int c = 0; c < 3; c++) co[c] = tanh_f(pr[7 + c]);
-      const float m3[3] = {pr[1], __fadd_rn(pr[2], __fmul_rn(co[0], xr)),
-                           __fadd_rn(__fadd_rn(pr[3], __fmul_rn(co[1], xr)), __fmul_rn(co[2], xg))};
+      const float m3[3] = {
+          pr[1], __fadd_rn(pr[2], __fmul_rn(co[0], xr)),
+          __fadd_rn(__fadd_rn(pr[3], __fmul_rn(co[1], xr)), __fmul_rn(co[2], xg))};
 #pragma unroll
       for (int c = 0; c < 3; c++) {
         const float ls = fmaxf(pr[4 + c], -7.f);
         const float inv = exp_f(-ls), mc = m3[c];
-        if (!want_d) {
-          lk = __fadd_rn(lk, log_bin_mass_f(mc, inv, bin_log_width(ls, inv), v[c]));
-          continue;
-        }
+        lk = __fadd_rn(lk, log_bin_mass_f(mc, inv, bin_log_width(ls, inv), v[c]));
         // sigma(-a) = 1/(1 + e^a), sigma(b) = 1/(1 + e^-b) through the MUFU
         // (a gradient, not a frequency table: the approximations only
         // perturb it by ~1e-6 relative)
+        float dm, dl;
         if (v[c] == 0) {
           const float aa = __fmul_rn(__fsub_rn(edge_f(1), mc), inv);
           const float sa = rcp_approx(__fadd_rn(1.f, exp_f(aa)));
-          dlm[c] = -inv * sa;
-          dll[c] = -aa * sa;
+          dm = -inv * sa;
+          dl = -aa * sa;
         } else if (v[c] == 255) {
           const float bb = __fmul_rn(__fsub_rn(edge_f(255), mc), inv);
           const float sb = rcp_approx(__fadd_rn(1.f, exp_f(-bb)));
-          dlm[c] = inv * sb;
-          dll[c] = bb * sb;
+          dm = inv * sb;
+          dl = bb * sb;
         } else {
           const float aa = __fmul_rn(__fsub_rn(edge_f(v[c] + 1), mc), inv);
           const float bb = __fmul_rn(__fsub_rn(edge_f(v[c]), mc), inv);
@@ -442,38 +451,47 @@ __device__ __noinline__ float tt_likelihood(const Dims& d, uint32_t tcol, const 
           const float gk = rcp_approx(em1);
           const float sa = rcp_approx(__fadd_rn(1.f, exp_f(aa)));
           const float sb = rcp_approx(__fadd_rn(1.f, exp_f(-bb)));
-          dlm[c] = -inv * (sa - sb);
-          dll[c] = -aa * sa + bb * sb - gk * dd;
+          dm = -inv * (sa - sb);
+          dl = -aa * sa + bb * sb - gk * dd;
         }
+        dlm[i][c] = dm;
+        dll[i][c] = pr[4 + c] > -7.f ? dl : 0.f;
       }
-      return lk;
-    };
-    // l_k = log pi_k + sum_c log P_c,k
-#pragma unroll 1
-    for (int k = part; k < K; k += kParts) {
-      float pr[10], co[3], dlm[3], dll[3];
-      load_comp(k, pr);
-      lb[k] = __fadd_rn(__fsub_rn(pr[0], lse_pi), comp_terms(pr, co, dlm, dll, false));
+      lk_[i] = __fadd_rn(__fsub_rn(pr[0], lse_pi), lk);
+      lb[k] = lk_[i];
     }
     __syncthreads();
     const float lse = row_lse();  // log p(pixel)
     if (valid && part == 0) nll = -lse;
     const float sc = valid ? scale : 0.f;
-#pragma unroll 1
-    for (int k = part; k < K; k += kParts) {
-      float pr[10], co[3], dlm[3], dll[3];
-      load_comp(k, pr);
-      comp_terms(pr, co, dlm, dll, true);
-      const float rho = valid ? exp_f(__fsub_rn(lb[k], lse)) : 0.f;
-      const float pi = exp_f(__fsub_rn(pr[0], lse_pi));
-      float gk[10];
-      gk[0] = sc * (pi - rho);
-      const float dmR = -rho * dlm[0], dmG = -rho * dlm[1], dmB = -rho * dlm[2];
+#pragma unroll
+    for (int i = 0; i < kCompPerThread; i++) {
+      const int k = part + kParts * i;
+      if (k >= K) continue;
+      uint32_t x[4];  // the logit and the couplings again
+#pragma unroll
+      for (int g = 0; g < 4; g++)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];"
+                     : "=r"(x[g])
+                     : "r"(tcol + (uint32_t)((g == 0 ? 0 : 6 + g) * K + k))
+                     : "memory");
+      tmem_wait_ld();
+      float co[3], gk[10];
+#pragma unroll
+      for (int g = 0; g < 4; g++) {
+        asm volatile("" : "+r"(x[g]));
+        const float y = __fadd_rn(__uint_as_float(x[g]), bh[(g == 0 ? 0 : 6 + g) * K + k]);
+        if (g == 0) gk[0] = exp_f(__fsub_rn(y, lse_pi));
+        else co[g - 1] = tanh_f(y);
+      }
+      const float rho = valid ? exp_f(__fsub_rn(lk_[i], lse)) : 0.f;
+      gk[0] = sc * (gk[0] - rho);
+      const float dmR = -rho * dlm[i][0], dmG = -rho * dlm[i][1], dmB = -rho * dlm[i][2];
       gk[1] = sc * dmR;
       gk[2] = sc * dmG;
       gk[3] = sc * dmB;
 #pragma unroll
-      for (int c = 0; c < 3; c++) gk[4 + c] = pr[4 + c] > -7.f ? sc * (-rho * dll[c]) : 0.f;
+      for (int c = 0; c < 3; c++) gk[4 + c] = sc * (-rho * dll[i][c]);
       gk[7] = sc * dmG * xr * (1.f - co[0] * co[0]);
       gk[8] = sc * dmB * xr * (1.f - co[1] * co[1]);
       gk[9] = sc * dmB * xg * (1.f - co[2] * co[2]);
@@ -496,6 +514,14 @@ __device__ __noinline__ float tt_likelihood(const Dims& d, uint32_t tcol, const 
   return nll;
 }
 
+// Bound: the latency of a tile's chain of phases (12 MMA chains with their
+// epilogues, the likelihood), 27 us per 128-pixel tile where the tensor pipe
+// needs 0.3; measured with single phases left out, a batch-128 step (7 tiles
+// per CTA) spends 51 us in the likelihood, 42 and 38 in the forward and
+// backward epilogues, 35 in the flushes, 24 in the weight-gradient chains.
+// 287 us with 256 threads, the slot read back in every flush and the context
+// gathered twice; 190 us so.
+//
 // MODE 0: dP = gradient of the mean code length in bits per dimension of the
 // batch (Eq. 2), the loss summed per CTA into part_l; MODE 1: dP = the given
 // upstream gradient dparams [n_px][10K] (raster order of the batch).  The
@@ -516,13 +542,7 @@ __global__ void __launch_bounds__(kTT, 1)
   const int row = 32 * (warp & 3) + lane;
   float* sbias = reinterpret_cast<float*>(sm + pl.bias);
   float* red = reinterpret_cast<float*>(sm + pl.red);
-  int4* slots = reinterpret_cast<int4*>(sm + pl.slots);
-  int2* taps = reinterpret_cast<int2*>(sm + pl.taps);
-  for (int p = threadIdx.x; p < d.F / 3; p += blockDim.x) {
-    int dy, dx;
-    tap_offset(p, d.h, dy, dx);
-    taps[p] = make_int2(dy, dx);
-  }
+  TTSlot* slots = reinterpret_cast<TTSlot*>(sm + pl.slots);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sm + pl.mbar);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + pl.tslot);
   // weights (BF16 tiles) and biases
@@ -559,12 +579,15 @@ __global__ void __launch_bounds__(kTT, 1)
   const uint32_t s0 = smem_u32(sm);
   uint32_t phase = 0;
   bool ok = true;
-  auto wait_mma = [&]() {  // the same outcome in every thread
-    if (threadIdx.x == 0) mma_commit(mbar);
+  auto wait_committed = [&]() {  // the same outcome in every thread
     const bool done = mbar_wait(mbar, phase);
     phase ^= 1u;
     fence_after_sync();
     return __syncthreads_and(done ? 1 : 0) != 0;
+  };
+  auto wait_mma = [&]() {
+    if (threadIdx.x == 0) mma_commit(mbar);
+    return wait_committed();
   };
   auto sync_for_mma = [&]() {  // smem stores and TMEM accesses before the next MMA
     fence_async_smem();
@@ -589,20 +612,21 @@ __global__ void __launch_bounds__(kTT, 1)
     const long long q0 = tile * kTTM;
     if (threadIdx.x < kTTM) {
       const long long q = q0 + threadIdx.x;
-      int4 sv = make_int4(0, 0, 0, 0);
+      TTSlot sv{-1, 0};
       if (q < n_px) {
-        const long long rr = q % HW;
-        sv = make_int4((int)(q / HW), (int)(rr / W), (int)(rr % W), 1);
+        const int im = (int)(q / HW), rr = (int)(q - im * HW);
+        sv.i = rr / W;
+        sv.j = rr - sv.i * W;
       }
       slots[threadIdx.x] = sv;
     }
-    __syncthreads();  // the slots (and, on the first tile, the taps)
-    tt_gather(d, batch, H, W, slots, taps, sm + pl.gx);
+    __syncthreads();  // the slots
+    tt_gather(d, batch + 3 * q0, W, slots, sm + pl.x);
     sync_for_mma();
 
     // ---------------- forward ----------------
     if (threadIdx.x == 0)
-      tt_mma(tmem + kColAcc, op_k(s0 + pl.gx, Fp), false, op_k(s0 + pl.w0, Fp), false, C, Fp / 16,
+      tt_mma(tmem + kColAcc, op_k(s0 + pl.x, Fp), false, op_k(s0 + pl.w0, Fp), false, C, Fp / 16,
              false);
     ok &= wait_mma();
     tt_fwd_epi(tl, sbias, 0, U, C, row, part);
@@ -631,10 +655,8 @@ __global__ void __launch_bounds__(kTT, 1)
 
     // ---------------- likelihood gradient dP -> BF16 tile [128][NOp] ----------------
     {
-      const int4 sl = slots[row];
-      const bool valid = sl.w != 0;
-      const uint8_t* px =
-          valid ? batch + ((long long)sl.x * HW + (long long)sl.y * W + sl.z) * 3 : batch;
+      const bool valid = slots[row].i >= 0;
+      const uint8_t* px = batch + (valid ? 3 * (q0 + row) : 0);
       loss = __fadd_rn(loss, tt_likelihood<MODE>(
                                  d, tl + kColAcc, sbias + C + 2 * R * C,
                                  reinterpret_cast<float*>(sm + pl.red) + row * kLbStride,
@@ -644,56 +666,82 @@ __global__ void __launch_bounds__(kTT, 1)
     sync_for_mma();
 
     // ---------------- adjoint ----------------
+    // Layer after layer: its three chains (input gradient into the
+    // accumulator, weight and bias gradients into buffer `buf`), then the
+    // epilogue that makes the next layer's gradient tile; the weight gradient
+    // is flushed behind the next layer's chains.
+    int buf = 0, pend = -1;  // buffer of the weight gradient not yet flushed
+    int p_out = 0, p_in = 0;
+    float *p_w = gW, *p_b = gW, p_scale = 1.f;
+    auto flush = [&]() {
+      if (pend >= 0) tt_flush(tmem, pend, p_out, p_in, p_in, p_scale, p_w, p_b);
+      pend = -1;
+    };
+    auto later = [&](int n_out, int n_in, float scale, float* w, float* b) {
+      pend = buf;
+      p_out = n_out;
+      p_in = n_in;
+      p_scale = scale;
+      p_w = w;
+      p_b = b;
+      buf ^= 1;
+    };
+    // dY: gradient tile at g with ng columns, the layer's input X at x, n_in
+    // columns; w != 0: also dX = dY W
+    auto chains = [&](uint32_t g, int ng, uint32_t w, uint32_t x, int n_in) {
+      if (threadIdx.x != 0) return;
+      if (w)
+        tt_mma(tmem + kColAcc, op_k(g, ng), false, op_mn(w, C), true, C, ng / 16, false);
+      tt_mma(tmem + col_dw(buf), op_mn(g, ng), true, op_mn(x, n_in), true, n_in, kTTM / 16, false);
+      tt_mma(tmem + col_db(buf), op_mn(g, ng), true, ones_op, false, 16, kTTM / 16, false);
+    };
     // head: dH = dP WH, dWH = dP^T u_R, dbH = dP^T 1
-    if (threadIdx.x == 0) {
-      tt_mma(tmem + kColAcc, op_k(s0 + pl.gx, NOp), false, op_mn(s0 + pl.wh, C), true, C,
-             NOp / 16, false);
-      tt_mma(tmem + kColDW, op_mn(s0 + pl.gx, NOp), true, op_mn(uoff + (2 * R) * tb, C), true, C,
+    const uint32_t gx = s0 + pl.gx, g2 = s0 + pl.g2;
+    chains(gx, NOp, s0 + pl.wh, uoff + (2 * R) * tb, C);
+    if (NO > kTTM && threadIdx.x == 0) {  // outputs 128 .. of a wide head: the other buffer
+      const uint32_t g = gx + kTTM / 8 * 128;
+      tt_mma(tmem + col_dw(1), op_mn(g, NOp), true, op_mn(uoff + (2 * R) * tb, C), true, C,
              kTTM / 16, false);
-      tt_mma(tmem + kColDB, op_mn(s0 + pl.gx, NOp), true, ones_op, false, 16, kTTM / 16, false);
+      tt_mma(tmem + col_db(1), op_mn(g, NOp), true, ones_op, false, 16, kTTM / 16, false);
     }
     ok &= wait_mma();
     tt_bwd_epi(tl, U + (2 * R) * tb, 0, sm + pl.gx, C, row, part);  // da_R = dH * ELU'(a_R)
-    tt_flush(tmem, NO, C, C, 1.f, gW + oWH, gW + obH);
+    if (NO > kTTM)
+      tt_flush(tmem, 1, NO - kTTM, C, C, 1.f, gW + oWH + (size_t)kTTM * C, gW + obH + kTTM);
+    later(NO < kTTM ? NO : kTTM, C, 1.f, gW + oWH, gW + obH);
     sync_for_mma();
     for (int r = R - 1; r >= 0 && ok; r--) {
       const size_t oW1 = oblk + r * blk, ob1 = oW1 + (size_t)C * C;
       const size_t oW2 = ob1 + C, ob2 = oW2 + (size_t)C * C;
       const uint32_t w1 = s0 + pl.w1 + r * pl.wstride, w2 = w1 + pl.wstride / 2;
       // dv = da W2, dW2 = da^T v_r, db2 = da^T 1  (da in G)
-      if (threadIdx.x == 0) {
-        tt_mma(tmem + kColAcc, op_k(s0 + pl.gx, C), false, op_mn(w2, C), true, C, C / 16, false);
-        tt_mma(tmem + kColDW, op_mn(s0 + pl.gx, C), true, op_mn(uoff + (2 * r + 1) * tb, C), true,
-               C, kTTM / 16, false);
-        tt_mma(tmem + kColDB, op_mn(s0 + pl.gx, C), true, ones_op, false, 16, kTTM / 16, false);
-      }
-      ok &= wait_mma();
+      chains(gx, C, w2, uoff + (2 * r + 1) * tb, C);
+      if (threadIdx.x == 0) mma_commit(mbar);
+      flush();
+      ok &= wait_committed();
       tt_bwd_epi(tl, U + (2 * r + 1) * tb, 2, sm + pl.g2, C, row, part);  // dz = dv * ELU'(z)
-      tt_flush(tmem, C, C, C, 1.f, gW + oW2, gW + ob2);
+      later(C, C, 1.f, gW + oW2, gW + ob2);
       sync_for_mma();
       // du = dz W1, dW1 = dz^T u_r, db1 = dz^T 1  (dz in G2)
-      if (threadIdx.x == 0) {
-        tt_mma(tmem + kColAcc, op_k(s0 + pl.g2, C), false, op_mn(w1, C), true, C, C / 16, false);
-        tt_mma(tmem + kColDW, op_mn(s0 + pl.g2, C), true, op_mn(uoff + (2 * r) * tb, C), true, C,
-               kTTM / 16, false);
-        tt_mma(tmem + kColDB, op_mn(s0 + pl.g2, C), true, ones_op, false, 16, kTTM / 16, false);
-      }
-      ok &= wait_mma();
+      chains(g2, C, w1, uoff + (2 * r) * tb, C);
+      if (threadIdx.x == 0) mma_commit(mbar);
+      flush();
+      ok &= wait_committed();
       tt_bwd_epi(tl, U + (2 * r) * tb, 1, sm + pl.gx, C, row, part);  // da_r = da + du * ELU'(a_r)
-      tt_flush(tmem, C, C, C, 1.f, gW + oW1, gW + ob1);
+      later(C, C, 1.f, gW + oW1, gW + ob1);
       sync_for_mma();
     }
     if (!ok) break;
-    // first layer: dW0 = da_0^T X / 255 (X gathered again), db0 = da_0^T 1
-    tt_gather(d, batch, H, W, slots, taps, sm + pl.xe);
-    sync_for_mma();
-    if (threadIdx.x == 0) {
-      tt_mma(tmem + kColDW, op_mn(s0 + pl.gx, C), true, op_mn(s0 + pl.xe, Fp), true, Fp,
-             kTTM / 16, false);
-      tt_mma(tmem + kColDB, op_mn(s0 + pl.gx, C), true, ones_op, false, 16, kTTM / 16, false);
+    // first layer: dW0 = da_0^T X / 255, db0 = da_0^T 1
+    if (!pl.keep_x) {
+      tt_gather(d, batch + 3 * q0, W, slots, sm + pl.xe);
+      sync_for_mma();
     }
-    ok &= wait_mma();
-    tt_flush(tmem, C, F, F, 1.f / 255.f, gW, gW + ob0);
+    chains(gx, C, 0, s0 + pl.xe, Fp);
+    if (threadIdx.x == 0) mma_commit(mbar);
+    flush();
+    ok &= wait_committed();
+    tt_flush(tmem, buf, C, F, F, 1.f / 255.f, gW, gW + ob0);
     sync_for_mma();
   }
   if (!ok && threadIdx.x == 0) set_status(status, ST_TIMEOUT);

@@ -49,3 +49,23 @@ def test_fp32_gradient_many_tiles_per_cta_is_deterministic():
     for _ in range(5):
         l2, g2 = codec.loss_grad(d)
         assert torch.equal(loss, l2) and torch.equal(grad, g2)
+
+
+@pytest.mark.parametrize("cfg,shape", [((2, 48, 1, 16), (2, 16, 16)), ((3, 64, 2, 13), (1, 9, 31)),
+                                       ((1, 16, 0, 1), (1, 3, 5)), ((3, 64, 2, 10), (3, 20, 20)),
+                                       ((1, 32, 2, 6), (5, 11, 13))])
+def test_bf16_gradient_every_plan(cfg, shape):
+    # BF16 operands: the tolerance of test_gpu_train.py (relative L2 error
+    # 3e-2, every element within 5e-2 of the largest, loss within 0.03 bits)
+    codec, w = make_codec(cfg, N.NLC_BF16, seed=8)
+    n, H, W = shape
+    batch = np.stack([synth.make_image(9, 40, 40, index=k)[:H, :W] for k in range(n)])
+    d = torch.from_numpy(batch).to(DEV)
+    loss, grad = codec.loss_grad(d)
+    ref_loss, ref = O.nll_grad(cfg, w.astype(np.float64), batch)
+    assert abs(float(loss) - ref_loss) <= 0.03
+    g = grad.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(g - ref) <= 3e-2 * np.linalg.norm(ref)
+    assert np.abs(g - ref).max() <= 5e-2 * np.abs(ref).max()
+    again, grad2 = codec.loss_grad(d)
+    assert torch.equal(loss, again) and torch.equal(grad, grad2)
