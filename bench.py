@@ -57,12 +57,12 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.44 MB written for
+# small case at 16 CTAs (1x1024^2: 5.72 MB read + 0.38 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.64
-TRAFFIC_SRC_SHA = "5856b340abd080beb5c2ca6fc09dd3385e37435a95fb530a31fc4ff604ea688d"
+TRAFFIC_B_PER_PX = 5.81
+TRAFFIC_SRC_SHA = "2c23f020c2a85e599fb5bc60eec511b7d9df2983aa5e170e66d2b2942f90bd3d"
 
 
 # the sources decode_kernel is compiled from

@@ -201,7 +201,7 @@ extern "C" int nlc_create(const nlc_model_cfg* cfg, const float* h_w, size_t n, 
     TRY_ALLOC(x->d_simt, simt_floats(x->d) * 4);
     TRY_ALLOC(x->d_umma, umma_halves(x->d) * 2);
     TRY_ALLOC(x->d_bias, bias_floats(x->d) * 4);
-    TRY_ALLOC(x->d_hash, 8);
+    TRY_ALLOC(x->d_hash, 8 * hash_words());
     TRY_ALLOC(x->d_status, 4);
     TRY_ALLOC(x->d_m, n * 4);
     TRY_ALLOC(x->d_v, n * 4);
@@ -216,6 +216,7 @@ extern "C" int nlc_create(const nlc_model_cfg* cfg, const float* h_w, size_t n, 
     if (rc) break;
     if ((e = cudaMemcpy(x->d_w, h_w, n * 4, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(x->d_status, 0, 4)) != cudaSuccess ||
+        (e = cudaMemset(x->d_hash, 0, 8 * hash_words())) != cudaSuccess ||
         (e = cudaMemset(x->d_m, 0, n * 4)) != cudaSuccess ||
         (e = cudaMemset(x->d_v, 0, n * 4)) != cudaSuccess) {
       rc = fail(NLC_ERR_CUDA, "initialisation failed: %s", cudaGetErrorString(e));

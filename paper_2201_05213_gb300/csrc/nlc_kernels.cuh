@@ -81,6 +81,8 @@ struct CodecBufs {
 // hash == nullptr: the packed copies only (the content hash is left as is)
 cudaError_t launch_repack(const Dims& d, const float* w, float* simt, uint16_t* umma, float* bias,
                           unsigned long long* hash, int n_w, cudaStream_t s);
+// hash: hash_words() words, zeroed once; the first receives the content hash.
+size_t hash_words();
 cudaError_t launch_hash(const Dims& d, const float* w, int n_w, unsigned long long* hash,
                         cudaStream_t s);
 
