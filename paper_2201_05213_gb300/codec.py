@@ -81,8 +81,11 @@ class Codec:
         return DecodePlan(self, sizes, patch, layout, schedule, outs)
 
     def forward(self, imgs, patch=0, params=True, bits=False, stream=None):
-        npx = sum(int(t.shape[0]) * int(t.shape[1]) for t in imgs)
         dev = imgs[0].device
+        return self._forward(N._images(imgs), dev, patch, params, bits, stream)
+
+    def _forward(self, imgs, dev, patch, params, bits, stream=None):
+        npx = imgs.pixels
         P = torch.empty((npx, 10 * self.cfg[3]), dtype=torch.float32, device=dev) if params else None
         B = torch.empty(npx, dtype=torch.float32, device=dev) if bits else None
         N.nlc_forward(self.ctx, imgs, patch, P, B, stream)
@@ -157,7 +160,7 @@ class DecodePlan:
 
 
 def _batch_images(batch):
-    return [batch[n] for n in range(batch.shape[0])]
+    return N._batch(batch) if batch.is_contiguous() else N._images(list(batch))
 
 
 class LocalModel(torch.autograd.Function):
@@ -169,7 +172,7 @@ class LocalModel(torch.autograd.Function):
     @staticmethod
     def forward(ctx, weights, codec, batch):
         N.nlc_load_weights(codec.ctx, weights.detach().contiguous())
-        P, _ = codec.forward(_batch_images(batch), 0)
+        P, _ = codec._forward(_batch_images(batch), batch.device, 0, True, False)
         ctx.codec, ctx.batch = codec, batch
         return P
 

@@ -270,10 +270,13 @@ extern "C" int nlc_weight_hash(nlc_ctx* x, uint64_t* h) {
 
 extern "C" int nlc_sync_status(nlc_ctx* x, nlc_stream stream) {
   if (!x) return fail(NLC_ERR_ARG, "ctx is NULL");
-  CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
+  // the copy runs behind the stream's work (to pageable memory: it returns when
+  // it is done), so one wait serves both; the word is cleared only when
+  // something was recorded
   int st = 0;
-  CUDA_TRY(cudaMemcpy(&st, x->d_status, 4, cudaMemcpyDeviceToHost));
-  CUDA_TRY(cudaMemset(x->d_status, 0, 4));
+  CUDA_TRY(cudaMemcpyAsync(&st, x->d_status, 4, cudaMemcpyDeviceToHost, (cudaStream_t)stream));
+  CUDA_TRY(cudaStreamSynchronize((cudaStream_t)stream));
+  if (st != 0) CUDA_TRY(cudaMemset(x->d_status, 0, 4));
   switch (st) {
     case 0: return NLC_OK;
     case ST_CAPACITY: return fail(NLC_ERR_CAPACITY, "output capacity exceeded");
