@@ -57,12 +57,12 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.72 MB read + 0.38 MB written for
+# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.22 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.81
-TRAFFIC_SRC_SHA = "2c23f020c2a85e599fb5bc60eec511b7d9df2983aa5e170e66d2b2942f90bd3d"
+TRAFFIC_B_PER_PX = 5.44
+TRAFFIC_SRC_SHA = "a5b1231e44faec61c59cacce20bc380041da1dca76b79ad1f4f5f43e9a68646e"
 
 
 # the sources decode_kernel is compiled from

@@ -78,31 +78,40 @@ struct F32Step {
   }
 };
 
-// acc[b][a] = sum over k < Kd (a multiple of 4), ascending, of w[k][b] in[k][a].
-// The next four inputs are read while the present ones are multiplied.
+// acc[b][a] = sum over k < Kd (a multiple of 4, at least 12), ascending, of
+// w[k][b] in[k][a].  The next U inputs are read while the present ones are
+// multiplied; blocks of few outputs read further ahead, to cover the reads'
+// latency with as many multiply-adds.
 template <int PX, int NB>
 __device__ __forceinline__ void f32_dot(const float* in, int ldm, int Kd, const float* w, int N,
                                         float (&acc)[NB][PX]) {
+  constexpr int U = PX * NB <= 4 ? 8 : 4;
 #pragma unroll
   for (int b = 0; b < NB; b++)
 #pragma unroll
     for (int a = 0; a < PX; a++) acc[b][a] = 0.f;
-  F32Step<4, PX, NB> s0, s1;
+  F32Step<U, PX, NB> s0, s1;
+  const int n = Kd / U * U;
   s0.load(in, ldm, w, N);
-  int k = 4;
+  int k = U;
 #pragma unroll 1
-  for (; k + 4 < Kd; k += 8) {
+  for (; k + U < n; k += 2 * U) {
     s1.load(in + k * ldm, ldm, w + k * N, N);
     s0.fma(acc);
-    s0.load(in + (k + 4) * ldm, ldm, w + (k + 4) * N, N);
+    s0.load(in + (k + U) * ldm, ldm, w + (k + U) * N, N);
     s1.fma(acc);
   }
-  if (k < Kd) {
+  if (k < n) {
     s1.load(in + k * ldm, ldm, w + k * N, N);
     s0.fma(acc);
     s1.fma(acc);
   } else {
     s0.fma(acc);
+  }
+  if (U > 4 && n < Kd) {
+    F32Step<4, PX, NB> s;
+    s.load(in + n * ldm, ldm, w + n * N, N);
+    s.fma(acc);
   }
 }
 
@@ -111,6 +120,7 @@ __device__ __forceinline__ void f32_dot(const float* in, int ldm, int Kd, const 
 // of pixel groups (a power of two).
 template <int PX, int NB>
 __device__ __noinline__ void f32_layers(Dims d, float* sm, int n, int MG) {
+  __builtin_assume(__isShared(sm));  // else every operand is a generic load
   const F32Plan pl = f32_plan(d);
   const int C = d.C, NOp = d.NOp, ldm = f32_ldm(n);
   const int mg = threadIdx.x & (MG - 1), ng = threadIdx.x / MG;
@@ -196,8 +206,9 @@ __device__ __forceinline__ void f32_gather(const Slot* slots, int n, const Dims 
     float v0 = 0.f, v1 = 0.f, v2 = 0.f;
     if (m < n) {
       const Slot s = slots[m];
-      int dy, dx;
-      tap_offset(p, h, dy, dx);
+      // tap_offset; p < 24, so the quotients by 3, 5 and 7 fit in a multiply
+      const int row = h == 1 ? (p * 43) >> 7 : h == 2 ? (p * 52) >> 8 : (p * 37) >> 8;
+      const int dy = row - h, dx = p - row * (2 * h + 1) - h;
       if (s.i + dy >= 0 && s.j + dx >= 0 && s.j + dx < s.Wu) {
         const uint8_t* px = s.px + (long long)dy * s.row_bytes + 3 * dx;
         const int a = kCoherent ? ld_cg_u8(px) : px[0], b = kCoherent ? ld_cg_u8(px + 1) : px[1],

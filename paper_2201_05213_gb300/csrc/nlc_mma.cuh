@@ -335,7 +335,7 @@ __device__ __noinline__ uint32_t net_layers(int n, bool win, uint32_t phase, lon
     }
     phase = (phase & ~(1u << LEVEL)) | (parity << LEVEL);
   }
-  // The head on all warps: every m-tile gets 16 / m-tiles of them.  The CTA
+  // The head: the m-tile's warps again (all 16 for a single m-tile).  The CTA
   // barrier is the last exchange and keeps P off the tiles it aliases.
   const int all_ok = __syncthreads_and(ok ? 1 : 0);
   if (pr) {
@@ -343,8 +343,9 @@ __device__ __noinline__ uint32_t net_layers(int n, bool win, uint32_t phase, lon
     pc[14] += c - ck;
     ck = c;
   }
-  const int mts = (n + 15) >> 4, wpm = kNetWarps / mts;
-  const int hm = warp / wpm, hs = warp % wpm;
+  const int mts = (n + 15) >> 4;
+  const int hlg = mts == 1 ? 4 : 3 - LEVEL;  // log2 of the warps per m-tile
+  const int wpm = 1 << hlg, hm = warp >> hlg, hs = warp & (wpm - 1);
   if (hm < mts) {
     const uint32_t wh = brow + (uint32_t)pl.wh;
     const uint32_t h = sb + (uint32_t)pl.h0 + (uint32_t)(16 * hm + (lane & 15)) * 16u +
@@ -519,14 +520,61 @@ __device__ __forceinline__ void gather_row_shear(const Slot& s, int dd, int h, i
                      [&](int kc) { return reinterpret_cast<uint4*>(X + kc * cs); });
 }
 
-// The decoder's tile, from its slots: a warp covers 8 pixels x 4 rows.
+// Columns 2 part, 2 part + 1 of one context row (masked tile): the same
+// features from the two or three words around their six bytes, for tiles of so
+// few pixels that a lane per row would leave most warps idle (8 pixels: one
+// warp with 250 instructions, 1.08 us; so 0.79).
+template <class Slot>
+__device__ __forceinline__ void gather_part(const Slot& s, int r, int part, int h, int F, int Fp,
+                                            uint16_t* X, int cs) {
+  const int w2 = 2 * h + 1, ncol = r < h ? w2 : h;
+  const int c0 = 2 * part;
+  if (r == h && part == 3)
+    for (int k = F; k < Fp; k++) X[(k >> 3) * cs + (k & 7)] = 0;
+  if (c0 >= ncol) return;
+  const int x0 = s.j - h + c0;  // image column (in the unit) of the first one
+  const bool row = s.i - h + r >= 0;
+  const bool in0 = row && x0 >= 0 && x0 < s.Wu;
+  const bool in1 = row && c0 + 1 < ncol && x0 + 1 >= 0 && x0 + 1 < s.Wu;
+  uint32_t w[3] = {0u, 0u, 0u};
+  uint32_t sh = 0;
+  if (in0 || in1) {
+    const uintptr_t lo = (uintptr_t)(s.px + (long long)(r - h) * s.row_bytes + 3 * (c0 - h));
+    const uintptr_t a = in0 ? lo : lo + 3, b = in1 ? lo + 6 : lo + 3;  // bytes inside the unit
+    const uintptr_t w0 = lo & ~(uintptr_t)3;
+    sh = 8u * (uint32_t)(lo & 3);
+#pragma unroll
+    for (int q = 0; q < 3; q++)
+      if (w0 + 4 * q + 4 > a && w0 + 4 * q < b) w[q] = ld_px_word<true>(w0 + 4 * q);
+  }
+  const uint32_t al[2] = {__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh)};
+  const int k0 = 3 * (r * w2 + c0);
+#pragma unroll
+  for (int q = 0; q < 6; q++) {
+    if (q >= 3 && c0 + 1 >= ncol) break;
+    const float x = (q < 3 ? in0 : in1) ? byte_input(al[q >> 2], q & 3) : 0.f;
+    const int k = k0 + q;
+    X[(k >> 3) * cs + (k & 7)] = __bfloat16_as_ushort(__float2bfloat16_rn(x));
+  }
+}
+
+// The decoder's tile, from its slots: a warp covers 8 pixels x 4 rows; up to
+// kFewPixels pixels (masked tile), 8 pixels x 4 column pairs of a row.
+constexpr int kFewPixels = 32;
 template <bool SHEAR>
 __device__ __noinline__ void net_gather(int slots, int n) {
   const NetSmem& t = net_smem();
   const Dims d = t.d;
   uint16_t* X = dec_at<uint16_t>(t.pl.x);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = lane >> 3, cs = 8 * t.rows;
+  const int cs = 8 * t.rows;
+  if (!SHEAR && n <= kFewPixels) {  // warp: row warp % 4 of the pixels 8 (warp / 4) ..
+    const int m = 8 * (warp >> 2) + (lane & 7), r = warp & 3;
+    if (m < n && r <= d.h)
+      gather_part(dec_at<DecSlot>(slots)[m], r, lane >> 3, d.h, d.F, d.Fp, X + 8 * m, cs);
+    return;
+  }
+  const int r = lane >> 3;
   for (int mb = 8 * warp; mb < n; mb += 8 * (int)(blockDim.x >> 5)) {
     const int m = mb + (lane & 7);
     if (r > d.h || m >= n) continue;

@@ -367,53 +367,31 @@ __device__ __forceinline__ float channel_setup(const CompState& cs, int K, int c
   return m;
 }
 
-// Decoder's symbol search for slot in [0, 2^16): s with cum_s <= slot <
-// cum_{s+1}, and those two values.  Round 1: lane gl evaluates cum at
-// b = B (gl + 1) (B = 256/GW; the last lane holds cum_256); the count c of
-// those <= slot locates s in [B c, B c + B).  Round 2: the B - 1 boundaries
-// inside, with the components split over the GW/B lanes that share one.
-template <int GW>
-__device__ __forceinline__ int cdf_search(const WarpScratch& ws, int nact, uint32_t slot, int gl,
+// Whole-warp symbol search for slot in [0, 2^16): s with cum_s <= slot <
+// cum_{s+1}, and those two values.  Two rounds of base 16; the lanes l and l +
+// 16 share boundary l's components (even and odd ones), so that a round of a
+// K = 10 mixture is one chunk of five terms per lane.  (31 boundaries with all
+// components each in the first round and 7 in the second took 14 % longer:
+// three chunks instead of two on the chain of every channel.)
+__device__ __forceinline__ int cdf_search(const WarpScratch& ws, int nact, uint32_t slot, int lane,
                                           uint32_t& c0, uint32_t& c1) {
-  constexpr int B = 256 / GW;
-  constexpr int P = GW / B;
   const unsigned full = 0xffffffffu;
-  uint32_t u1 = 65536u;
-  if (gl < GW - 1) {
-    const int b = B * (gl + 1);
-    u1 = cum_fix(cdf_fix<GW == 32>(ws, nact, edge_f(b), 0, 1), b);
-  }
-  const int c = __popc(grp_ballot<GW>(u1 <= slot));
-  const int j = gl % B, part = gl / B;
-  const int b2 = B * c + j + 1;
-  uint32_t F2 = 0;
-  if (j < B - 1) F2 = cdf_fix<GW == 32>(ws, nact, edge_f(b2), part, P);
-#pragma unroll
-  for (int o = B; o < GW; o <<= 1) F2 += __shfl_xor_sync(full, F2, o, GW);
-  const uint32_t top = __shfl_sync(full, u1, c, GW);  // cum_{B (c+1)}
-  const uint32_t u2 = j < B - 1 ? cum_fix(F2, b2) : top;
-  const int c2 = __popc(grp_ballot<GW>(part == 0 && u2 <= slot));
-  c1 = __shfl_sync(full, u2, c2, GW);
-  const uint32_t lo2 = __shfl_sync(full, u2, c2 > 0 ? c2 - 1 : 0, GW);
-  const uint32_t lo1 = __shfl_sync(full, u1, c > 0 ? c - 1 : 0, GW);
+  const int j = lane & 15, half = lane >> 4;
+  uint32_t F = cdf_fix<true>(ws, nact, edge_f(16 * (j + 1)), half, 2);
+  F += __shfl_xor_sync(full, F, 16);
+  const uint32_t u1 = j < 15 ? cum_fix(F, 16 * (j + 1)) : 65536u;
+  const int c = __popc(__ballot_sync(full, u1 <= slot) & 0xFFFFu);
+  const int b2 = 16 * c + j + 1;
+  F = cdf_fix<true>(ws, nact, edge_f(b2), half, 2);
+  F += __shfl_xor_sync(full, F, 16);
+  const uint32_t top = __shfl_sync(full, u1, c);  // cum_{16 (c+1)}
+  const uint32_t u2 = j < 15 ? cum_fix(F, b2) : top;
+  const int c2 = __popc(__ballot_sync(full, u2 <= slot) & 0xFFFFu);
+  c1 = __shfl_sync(full, u2, c2);
+  const uint32_t lo2 = __shfl_sync(full, u2, c2 > 0 ? c2 - 1 : 0);
+  const uint32_t lo1 = __shfl_sync(full, u1, c > 0 ? c - 1 : 0);
   c0 = c2 > 0 ? lo2 : (c > 0 ? lo1 : 0u);
-  return B * c + c2;
-}
-
-// Encoder's pair cum_v, cum_{v+1}: lanes of even / odd gl evaluate b = v /
-// v + 1 over components gl/2 and gl/2 + GW/2 (K <= 16: every component once).
-template <int GW>
-__device__ __forceinline__ void cdf_pair(const WarpScratch& ws, int v, int gl, uint32_t& c0,
-                                         uint32_t& c1) {
-  const unsigned full = 0xffffffffu;
-  const int b = v + (gl & 1);
-  const float e = edge_f(b);
-  uint32_t F = cdf_term(e, ws.cp[gl >> 1]) + cdf_term(e, ws.cp[(gl >> 1) + GW / 2]);
-#pragma unroll
-  for (int o = 2; o < GW; o <<= 1) F += __shfl_xor_sync(full, F, o, GW);
-  const uint32_t u = cum_fix(F, b);
-  c0 = __shfl_sync(full, u, 0, GW);
-  c1 = __shfl_sync(full, u, 1, GW);
+  return 16 * c + c2;
 }
 
 // Symbol s with cum_s <= slot < cum_{s+1} in an explicit table.

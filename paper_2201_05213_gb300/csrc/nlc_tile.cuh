@@ -150,27 +150,98 @@ struct GroupRansDec {
   }
 };
 
-// Encodes symbols k = nsym-1 .. 0 (packed start | freq << 16) ending at
-// slot_end; returns the stream length.  Layout: 4-byte big-endian final
-// state, then the emitted bytes in reverse emission order.
-template <class Get>
-__device__ __forceinline__ int rans_encode_stream(Get get, long long nsym, uint8_t* slot_end) {
-  uint8_t* w = slot_end;
-  uint32_t x = kRansL;
-  for (long long k = nsym - 1; k >= 0; k--) {
-    const uint32_t e = get(k);
-    const uint32_t start = e & 0xFFFFu, f = e >> 16;
-    const uint32_t xmax = ((kRansL >> 16) << 8) * f;
-    while (x >= xmax) {
-      *--w = (uint8_t)(x & 0xFFu);
-      x >>= 8;
-    }
-    x = ((x / f) << 16) + (x % f) + start;
+// Reciprocal of a symbol's frequency (packed start | freq << 16) for rans_put.
+__device__ __forceinline__ uint32_t rans_recip(uint32_t e) { return 0xFFFFFFFFu / (e >> 16); }
+
+// One rANS step: the bytes that leave the state go downwards from w.  The
+// quotient x / f is umulhi(x, m) with m = floor((2^32 - 1) / f), or one more:
+// m > 2^32 / f - 1 - 1/f, so the product is short by less than x / 2^31 <= 1
+// (x < 2^31), and one comparison corrects it.  m does not depend on the state,
+// so the states' chain holds no division.
+__device__ __forceinline__ void rans_put(uint32_t e, uint32_t m, uint32_t& x, uint8_t*& w,
+                                         bool store = true) {
+  const uint32_t start = e & 0xFFFFu, f = e >> 16;
+  const uint32_t xmax = ((kRansL >> 16) << 8) * f;
+  while (x >= xmax) {
+    --w;
+    if (store) *w = (uint8_t)(x & 0xFFu);
+    x >>= 8;
   }
+  uint32_t q = __umulhi(x, m);
+  uint32_t r = x - q * f;
+  if (r >= f) {
+    q++;
+    r -= f;
+  }
+  x = (q << 16) + r + start;
+}
+
+// The final state, 4 bytes big-endian, in front of the emitted bytes.
+__device__ __forceinline__ void rans_flush(uint32_t x, uint8_t*& w) {
   *--w = (uint8_t)x;
   *--w = (uint8_t)(x >> 8);
   *--w = (uint8_t)(x >> 16);
   *--w = (uint8_t)(x >> 24);
+}
+
+// Encodes symbols k = nsym-1 .. 0 (packed start | freq << 16) ending at
+// slot_end by one thread; returns the stream length.  Layout: 4-byte
+// big-endian final state, then the emitted bytes in reverse emission order.
+// The next four symbols are read, and the present ones' reciprocals taken,
+// ahead of the chain.
+template <class Get>
+__device__ __forceinline__ int rans_encode_stream(Get get, long long nsym, uint8_t* slot_end) {
+  uint8_t* w = slot_end;
+  uint32_t x = kRansL;
+  constexpr int U = 4;
+  long long k = nsym;
+  uint32_t n[U] = {};
+#pragma unroll
+  for (int i = 0; i < U; i++)
+    if (k > i) n[i] = get(k - 1 - i);
+  for (; k >= U; k -= U) {
+    uint32_t e[U], m[U];
+#pragma unroll
+    for (int i = 0; i < U; i++) {
+      e[i] = n[i];
+      if (k - U > i) n[i] = get(k - U - 1 - i);
+    }
+#pragma unroll
+    for (int i = 0; i < U; i++) m[i] = rans_recip(e[i]);
+#pragma unroll
+    for (int i = 0; i < U; i++) rans_put(e[i], m[i], x, w);
+  }
+#pragma unroll
+  for (int i = 0; i < U; i++)
+    if (k > i) rans_put(n[i], rans_recip(n[i]), x, w);
+  rans_flush(x, w);
+  return (int)(slot_end - w);
+}
+
+// The same by a warp: the lanes read 32 symbols and take their reciprocals at
+// once, then all follow the chain (lane 0 stores).
+template <class Get>
+__device__ __forceinline__ int rans_encode_warp(Get get, long long nsym, uint8_t* slot_end) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  uint8_t* w = slot_end;
+  uint32_t x = kRansL;
+  uint32_t n = lane < nsym ? get(nsym - 1 - lane) : 0x10000u;
+  for (long long k = nsym; k > 0; k -= 32) {
+    const uint32_t e = n, m = rans_recip(e);
+    n = k - 32 > lane ? get(k - 33 - lane) : 0x10000u;
+    const int c = k < 32 ? (int)k : 32;
+    if (c == 32) {
+#pragma unroll 8
+      for (int i = 0; i < 32; i++)
+        rans_put(__shfl_sync(full, e, i), __shfl_sync(full, m, i), x, w, lane == 0);
+    } else {
+      for (int i = 0; i < c; i++)
+        rans_put(__shfl_sync(full, e, i), __shfl_sync(full, m, i), x, w, lane == 0);
+    }
+  }
+  if (lane == 0) rans_flush(x, w);
+  else w -= 4;
   return (int)(slot_end - w);
 }
 
