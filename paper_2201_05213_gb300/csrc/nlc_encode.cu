@@ -6,10 +6,10 @@
 
 namespace nlc {
 
-// Warps per CTA of the BF16 kernel: 12 leave each thread 168 registers, which
-// the 64-channel network needs (two sets of 32 accumulators and 16 fragments);
-// with 16 warps of 128 registers it spills.
-constexpr int kPxWarps = 12;
+// Warps per CTA of the BF16 kernel.  Four per scheduler at 128 registers (16
+// to 24 bytes spilled) hide the chains better than three at 168: 5.5 against
+// 6.1 ms for 12.6 M pixels; 14 leave the schedulers uneven (6.3 ms).
+constexpr int kPxWarps = 16;
 
 struct PxArgs {
   DeviceModel m;
@@ -54,7 +54,13 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
   PxSlot* slots = reinterpret_cast<PxSlot*>(own + pl.x_bytes);
   const uint32_t sb = smem_u32(smem), xa = smem_u32(own);
   const float* bh = bias + 8 * NT8 * (1 + 2 * d.R);
+  uint32_t* row = reinterpret_cast<uint32_t*>(smem + pl.row);
+  float* hbias = reinterpret_cast<float*>(smem + pl.hbias);
+  static_assert(PxHead<KI>::kBytes <= kPxTables, "the tables' place");
   __syncthreads();
+  px_head_tables<NT8, KI>(d, bh, row, hbias);
+  __syncthreads();
+  const uint32_t wh = sb + (uint32_t)pl.wh;
   const long long groups = (a.n_px + kPxRows - 1) / kPxRows;
   int hint = 0;
   for (long long grp = (long long)blockIdx.x * nw + warp; grp < groups;
@@ -86,20 +92,19 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
         for (int c = 0; c < 3; c++) v[r][c] = __ldg(px + c);
       }
     }
-    constexpr int p0[3] = {0, 1, 4}, p1[3] = {2, 5, 7}, p2[4] = {3, 6, 8, 9};
     if constexpr (ENC) {
       QuadState<KI> st[2];
       uint32_t e[2][3];
       {
         float w[2][3 * KI];
-        px_head<NT8, KI, 3>(d, pl, sb, bh, f, p0, w);
+        px_head<NT8, KI, 0>(wh, row, hbias, f, w);
 #pragma unroll
         for (int r = 0; r < 2; r++) {
           auto P = [&](int p, int i) { return w[r][(p == 0 ? 0 : p == 1 ? 1 : 2) * KI + i]; };
           quad_init<KI>(P, K, q, st[r]);
           e[r][0] = enc_channel<0, KI>(P, K, q, v[r], st[r]);
         }
-        px_head<NT8, KI, 3>(d, pl, sb, bh, f, p1, w);
+        px_head<NT8, KI, 1>(wh, row, hbias, f, w);
 #pragma unroll
         for (int r = 0; r < 2; r++)
           e[r][1] = enc_channel<1, KI>(
@@ -107,7 +112,7 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
               v[r], st[r]);
       }
       float w[2][4 * KI];
-      px_head<NT8, KI, 4>(d, pl, sb, bh, f, p2, w);
+      px_head<NT8, KI, 2>(wh, row, hbias, f, w);
 #pragma unroll
       for (int r = 0; r < 2; r++)
         e[r][2] = enc_channel<2, KI>(
@@ -125,14 +130,14 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
       const bool in[2] = {q0 + g < a.n_px, q0 + g + 8 < a.n_px};
       if (a.params) {
         const int NO = d.NO;
-        const uint32_t wh = sb + (uint32_t)pl.wh + (lane & 7) * 16u;
+        const uint32_t wr = wh + (lane & 7) * 16u;
 #pragma unroll 1
         for (int j = 0; 8 * j < NO; j++) {
           uint32_t w[NT8];
-          load_b<NT8 / 2>(wh + (uint32_t)j * (128u * NT8), w);
-          float c[4] = {0.f, 0.f, 0.f, 0.f};
+          load_b<NT8 / 2>(wr + (uint32_t)j * (128u * NT8), w);
+          float c[4];
 #pragma unroll
-          for (int s = 0; s < NT8 / 2; s++) mma_16816(c, f[s], w[2 * s], w[2 * s + 1]);
+          for (int s = 0; s < NT8 / 2; s++) mma_step(s, c, f[s], w[2 * s], w[2 * s + 1]);
           const int col = 8 * j + 2 * q;
           if (col < NO) {
             const float2 b = *reinterpret_cast<const float2*>(bh + col);
@@ -148,14 +153,14 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
         QuadState<KI> st[2];
         {
           float w[2][3 * KI];
-          px_head<NT8, KI, 3>(d, pl, sb, bh, f, p0, w);
+          px_head<NT8, KI, 0>(wh, row, hbias, f, w);
 #pragma unroll
           for (int r = 0; r < 2; r++) {
             auto P = [&](int p, int i) { return w[r][(p == 0 ? 0 : p == 1 ? 1 : 2) * KI + i]; };
             quad_init<KI>(P, K, q, st[r]);
             quad_loglik<0, KI>(P, K, q, v[r], st[r].lw);
           }
-          px_head<NT8, KI, 3>(d, pl, sb, bh, f, p1, w);
+          px_head<NT8, KI, 1>(wh, row, hbias, f, w);
 #pragma unroll
           for (int r = 0; r < 2; r++)
             quad_loglik<1, KI>(
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
                 v[r], st[r].lw);
         }
         float w[2][4 * KI];
-        px_head<NT8, KI, 4>(d, pl, sb, bh, f, p2, w);
+        px_head<NT8, KI, 2>(wh, row, hbias, f, w);
 #pragma unroll
         for (int r = 0; r < 2; r++) {
           quad_loglik<2, KI>(

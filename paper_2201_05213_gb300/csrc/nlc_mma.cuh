@@ -132,6 +132,21 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// The first K step: C = 0 (no registers to clear).
+__device__ __forceinline__ void mma_16816_first(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                                uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+// K step s of a chain.
+__device__ __forceinline__ void mma_step(int s, float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
+  if (s == 0) mma_16816_first(c, a, b0, b1);
+  else mma_16816(c, a, b0, b1);
+}
+
 // Two FP32 operations in one instruction, each rounded as its scalar form.
 __device__ __forceinline__ void add2(float& a, float& b, float x, float y) {
   asm("{\n.reg .b64 p, q;\nmov.b64 p, {%0, %1};\nmov.b64 q, {%2, %3};\n"
@@ -309,13 +324,9 @@ __device__ __noinline__ uint32_t net_layers(int n, bool win, uint32_t phase, lon
     auto hidden = [&](uint32_t h) {
       load_a(h);
 #pragma unroll
-      for (int i = 0; i < TP; i++)
-#pragma unroll
-        for (int e = 0; e < 4; e++) acc[i][e] = 0.f;
-#pragma unroll
       for (int s = 0; s < KS; s++)
 #pragma unroll
-        for (int i = 0; i < TP; i++) mma_16816(acc[i], a[s], w[i][2 * s], w[i][2 * s + 1]);
+        for (int i = 0; i < TP; i++) mma_step(s, acc[i], a[s], w[i][2 * s], w[i][2 * s + 1]);
     };
     uint32_t wl = brow + (uint32_t)pl.w1;
     epilogue(bias, IntC<0>{}, o0);
@@ -365,13 +376,11 @@ __device__ __noinline__ uint32_t net_layers(int n, bool win, uint32_t phase, lon
       for (int i = 0; i < HG; i++) {
         const int j = j0 + i * wpm;
         load_b<KS>(wh + (uint32_t)(j < nht ? j : j0) * (128u * NT8), w[i]);
-#pragma unroll
-        for (int e = 0; e < 4; e++) acc[i][e] = 0.f;
       }
 #pragma unroll
       for (int s = 0; s < KS; s++)
 #pragma unroll
-        for (int i = 0; i < HG; i++) mma_16816(acc[i], a[s], w[i][2 * s], w[i][2 * s + 1]);
+        for (int i = 0; i < HG; i++) mma_step(s, acc[i], a[s], w[i][2 * s], w[i][2 * s + 1]);
 #pragma unroll
       for (int i = 0; i < HG; i++) {
         const int j = j0 + i * wpm;

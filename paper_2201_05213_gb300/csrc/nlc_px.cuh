@@ -8,11 +8,11 @@
 // head's weight rows are read in an order that leaves every lane with whole
 // mixture components of its two pixels, so the coding starts from registers
 // too.  Only the context tile (16 pixels) passes through shared memory, where
-// the weights stay for the CTA's lifetime.  Bound: instruction issue (57 % of
-// the slots, 310 warp instructions per pixel; MUFU 25 %, tensor pipe 21 %).
-// Measured, the tables of 12.6 M pixels (h = 3, C = 64, R = 2, K = 10): 18.6 ms
-// with one 128-pixel tcgen05 tile at a time per SM and 16 lanes per pixel, 5.6
-// ms so.
+// the weights stay for the CTA's lifetime.  Bound: instruction issue (57 %
+// of the slots at twelve warps, 310 warp instructions per pixel; MUFU 25 %,
+// tensor pipe 21 %).  Measured, the tables of 12.6 M pixels (h = 3, C = 64, R
+// = 2, K = 10): 18.6 ms with one 128-pixel tcgen05 tile at a time per SM and 16
+// lanes per pixel, 4.8 ms so.
 #pragma once
 
 #include "nlc_mma.cuh"
@@ -32,10 +32,12 @@ struct alignas(16) PxSlot {
   long long out;      // forward: index of its outputs (images in order, raster)
 };
 
-// Byte offsets: the weights and biases, then per warp a context tile and slots.
+// Byte offsets: the weights and biases, the head's tables, then per warp a
+// context tile and slots.
 struct PxPlan {
-  int w0, w1, wh, w0s, bias, warp0, x_bytes, per_warp;
+  int w0, w1, wh, w0s, bias, row, hbias, warp0, x_bytes, per_warp;
 };
+constexpr int kPxTables = 20 * 64;  // bytes of the head's tables (kTiles <= 20)
 __host__ __device__ inline PxPlan px_plan(const Dims& d) {
   const TcPlan tp = tc_plan(d);
   PxPlan p;
@@ -44,7 +46,9 @@ __host__ __device__ inline PxPlan px_plan(const Dims& d) {
   p.wh = tp.wh;
   p.w0s = tp.w0s;
   p.bias = tp.bias;
-  p.warp0 = align_up(tp.bias + (int)(d.C + 2 * d.R * d.C + d.NOp) * 4, 128);
+  p.row = align_up(tp.bias + (int)(d.C + 2 * d.R * d.C + d.NOp) * 4, 16);
+  p.hbias = p.row + kPxTables / 2;
+  p.warp0 = align_up(p.row + kPxTables, 128);
   p.x_bytes = kPxRows * 2 * (d.shear ? (d.h + 1) * d.Fsp : d.Fp);
   p.per_warp = align_up(p.x_bytes + kPxRows * (int)sizeof(PxSlot), 128);
   return p;
@@ -144,13 +148,9 @@ __device__ __forceinline__ void px_hidden(const Dims& d, const PxPlan& pl, uint3
 #pragma unroll
       for (int i = 0; i < 2; i++) load_b<KS>(wl + (uint32_t)(j + i) * (128u * NT8), w[i]);
 #pragma unroll
-      for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int e = 0; e < 4; e++) acc[j + i][e] = 0.f;
-#pragma unroll
       for (int s = 0; s < KS; s++) {
-        mma_16816(acc[j], a[s], w[0][2 * s], w[0][2 * s + 1]);
-        mma_16816(acc[j + 1], a[s], w[1][2 * s], w[1][2 * s + 1]);
+        mma_step(s, acc[j], a[s], w[0][2 * s], w[0][2 * s + 1]);
+        mma_step(s, acc[j + 1], a[s], w[1][2 * s], w[1][2 * s + 1]);
       }
     }
     wl += kWBytes;
@@ -181,46 +181,68 @@ __device__ __forceinline__ void px_hidden(const Dims& d, const PxPlan& pl, uint3
   }
 }
 
-// The head outputs of NP parameter groups (ps[0 .. NP): 0 logits, 1..3
-// locations, 4..6 log-scales, 7..9 couplings) as whole components per lane:
-// v[r][p * KI + i] = output ps[p] of component q + 4 i of the lane's pixel r
-// (rows g, g + 8).  Column 2 q + e of the t-th tile is value 2 t + e of lane
-// q, so the tile's weight rows are gathered accordingly (ldmatrix takes a row
-// address per lane); components past K read a zero row, which exists because
-// 10 K is then no multiple of 16.
-template <int NT8, int KI, int NP>
-__device__ __forceinline__ void px_head(const Dims& d, const PxPlan& pl, uint32_t sb,
-                                        const float* bh, const uint32_t (&a)[NT8 / 2][4],
-                                        const int (&ps)[NP], float (&v)[2][NP * KI]) {
-  constexpr int KS = NT8 / 2, S = NP * KI;
-  const int lane = threadIdx.x & 31, q = lane & 3, K = d.K;
-  auto row_of = [&](int slot, int qq) {  // weight row of value `slot` of quad lane qq
-    const int k = qq + 4 * (slot % KI);
-    return slot < S && k < K ? ps[slot / KI < NP ? slot / KI : 0] * K + k : d.NO;
-  };
+// The head as the quads want it.  Its outputs are taken in three groups (one
+// per channel: logits, location, log-scale; location, log-scale, coupling;
+// location, log-scale, two couplings), each as whole components per lane:
+// value p * KI + i of lane q is the group's p-th output of component q + 4 i.
+// Column 2 q + e of a group's t-th tile is value 2 t + e of lane q, so the
+// tile's weight rows are gathered accordingly (ldmatrix takes a row address
+// per lane); components past K read a zero row, which exists because 10 K is
+// then no multiple of 16.  Which rows and biases these are depends on the model
+// alone: they are tables in shared memory, filled once per CTA.
+template <int KI>
+struct PxHead {
+  static constexpr int kTiles = 2 * ((3 * KI + 1) / 2) + 2 * KI;  // 8-column tiles of the groups
+  static constexpr int kBytes = kTiles * (8 * 4 + 8 * 4);
+  // first tile of channel ch's group
+  __host__ __device__ static constexpr int first(int ch) { return ch * ((3 * KI + 1) / 2); }
+};
+// Output (0 logits, 1..3 locations, 4..6 log-scales, 7..9 couplings) p of
+// channel ch's group.
+__device__ __forceinline__ int px_output(int ch, int p) {
+  return ch == 0 ? (p == 0 ? 0 : p == 1 ? 1 : 4)
+                 : ch == 1 ? (p == 0 ? 2 : p == 1 ? 5 : 7)
+                           : (p == 0 ? 3 : p == 1 ? 6 : 6 + p);
+}
+// row[t][r]: byte offset (from the head's weights) of row r of tile t; bias[t][2 q + e].
+template <int NT8, int KI>
+__device__ __forceinline__ void px_head_tables(const Dims& d, const float* bh, uint32_t* row,
+                                               float* bias) {
+  using H = PxHead<KI>;
+  for (int i = threadIdx.x; i < 8 * H::kTiles; i += blockDim.x) {
+    const int t = i >> 3, q = (i & 7) >> 1, e = i & 1;
+    const int ch = t >= H::first(2) ? 2 : t >= H::first(1) ? 1 : 0;
+    const int slot = 2 * (t - H::first(ch)) + e, np = ch == 2 ? 4 : 3;
+    const int k = q + 4 * (slot % KI);
+    int n = slot < np * KI && k < d.K ? px_output(ch, slot / KI) * d.K + k : d.NO;
+    if (n >= d.NOp) n = 0;  // a value that no lane uses: any row will do
+    row[i] = (uint32_t)((n >> 3) * NT8) * 128u + (uint32_t)(n & 7) * 16u;
+    bias[i] = bh[n];
+  }
+}
+
+// Channel CH's group: v[r][value] of the lane's pixel r (rows g, g + 8).
+template <int NT8, int KI, int CH>
+__device__ __forceinline__ void px_head(uint32_t wh, const uint32_t* row, const float* bias,
+                                        const uint32_t (&a)[NT8 / 2][4],
+                                        float (&v)[2][(CH == 2 ? 4 : 3) * KI]) {
+  constexpr int KS = NT8 / 2, S = (CH == 2 ? 4 : 3) * KI, T0 = PxHead<KI>::first(CH);
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int t = 0; t < (S + 1) / 2; t++) {
-    const int qr = (lane & 7) >> 1;
-    const int r0 = row_of(2 * t, qr), r1 = row_of(2 * t + 1, qr);
-    const int n = (lane & 1) ? r1 : r0;
-    // rows that no lane uses may lie past the matrix: any row of it will do
-    const int nr = n < d.NOp ? n : 0;
-    const uint32_t w0 = sb + (uint32_t)pl.wh + (uint32_t)((nr >> 3) * NT8) * 128u +
-                        (uint32_t)(nr & 7) * 16u;
     uint32_t w[2 * KS];
-    load_b<KS>(w0, w);
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
+    load_b<KS>(wh + row[8 * (T0 + t) + (lane & 7)], w);
+    float c[4];
 #pragma unroll
-    for (int s = 0; s < KS; s++) mma_16816(c, a[s], w[2 * s], w[2 * s + 1]);
-#pragma unroll
-    for (int e = 0; e < 2; e++) {
-      const int slot = 2 * t + e;
-      if (slot < S) {
-        const int nb = row_of(slot, q);
-        const float b = bh[nb < d.NOp ? nb : 0];
-        v[0][slot] = __fadd_rn(c[e], b);
-        v[1][slot] = __fadd_rn(c[2 + e], b);
-      }
+    for (int s = 0; s < KS; s++) mma_step(s, c, a[s], w[2 * s], w[2 * s + 1]);
+    const float2 b = *reinterpret_cast<const float2*>(bias + 8 * (T0 + t) + 2 * (lane & 3));
+    add2(c[0], c[1], b.x, b.y);
+    add2(c[2], c[3], b.x, b.y);
+    v[0][2 * t] = c[0];
+    v[1][2 * t] = c[2];
+    if (2 * t + 1 < S) {
+      v[0][2 * t + 1] = c[1];
+      v[1][2 * t + 1] = c[3];
     }
   }
 }
