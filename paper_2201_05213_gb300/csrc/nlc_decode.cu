@@ -19,6 +19,13 @@ static int decode_rows(const Dims& d, int n_units, bool win) {
                                                                               : kTileMax / 2;
 }
 
+// The limit is the function's, not a launch's: were it set to each batch's own
+// need, a plan made for a small batch would take it from an earlier plan's
+// larger one.
+static cudaError_t allow_smem(const void* fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 size_t decode_smem_bytes(const Dims& d, int n_units, bool win) {
   return dec_carve(d, n_units, decode_rows(d, n_units, win), win, nullptr);
 }
@@ -45,9 +52,7 @@ int decode_max_grid(const DeviceModel& m, int n_units, int sm_count, bool sample
   int best = -1;
   for (int prof = 0; prof < (sample ? 1 : 2); prof++) {
     const void* fn = decode_fn(m.d.prec, sample, win, prof != 0);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return 0;
+    if (allow_smem(fn) != cudaSuccess) return 0;
     int per = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, decode_threads_of(m.d.prec),
                                                       smem) != cudaSuccess)
@@ -92,8 +97,7 @@ cudaError_t launch_decode(const DeviceModel& m, const CodecBufs& b, const uint8_
   const void* fn = decode_fn(m.d.prec, false, win, b.prof != nullptr);
   const int nt = decode_threads_of(m.d.prec);
   if (set_attr &&
-      (e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-          cudaSuccess)
+      (e = allow_smem(fn)) != cudaSuccess)
     return e;
   a.seed = 0;
   void* args[] = {&a};
@@ -129,9 +133,7 @@ cudaError_t launch_sample(const DeviceModel& m, const CodecBufs& b, int sched, i
   const size_t smem = decode_smem_bytes(m.d, b.n_units, win);
   const void* fn = decode_fn(m.d.prec, true, win);
   const int nt = decode_threads_of(m.d.prec);
-  if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_smem(fn)) != cudaSuccess) return e;
   void* args[] = {&a};
   if (grid > 1) return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(nt), args, smem, s);
   return cudaLaunchKernel(fn, dim3(1), dim3(nt), args, smem, s);

@@ -70,3 +70,19 @@ def test_wide_heads_match_the_oracle(K):
     P, _ = codec.forward([to_dev(img)], 0)
     ref = O.forward_image(cfg, w, img).reshape(-1, 10 * K)
     assert np.abs(P.cpu().numpy().astype(np.float64) - ref).max() <= 2e-2
+
+
+def test_a_small_plan_leaves_an_earlier_large_one_usable():
+    # the kernels' shared-memory limit is set per function: a later plan of a
+    # small batch must not lower it below an earlier plan's need
+    codec, _ = make_codec((1, 32, 1, 5), N.NLC_BF16, seed=3)
+    d = torch.cat([to_dev(i).reshape(-1, 3) for i in images(23, [(64, 64)])])
+    many = [d[5 * k:5 * k + 9].reshape(1, 9, 3).contiguous() for k in range(700)]
+    data, offs = codec.compress(many, 0, N.NLC_LAYOUT_ROW)
+    large = codec.plan([(1, 9)] * 700, 0, N.NLC_LAYOUT_ROW)
+    small = codec.plan([(1, 9)], 0, N.NLC_LAYOUT_ROW)
+    large.run(data, offs)
+    codec.check()
+    assert all(torch.equal(a, b) for a, b in zip(large.outs, many))
+    small.close()
+    large.close()
