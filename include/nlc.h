@@ -20,13 +20,13 @@
  *     library owns only the context and a device workspace that it grows on
  *     demand (so the first call with a larger batch allocates).
  *   - Images are uint8 H x W x 3 (RGB), C-contiguous, row stride 3 W bytes.
- *     Kernels read image buffers (the inputs of the compress calls and of
- *     nlc_forward, and the outputs of the decode calls, whose decoded pixels
- *     are the context of later ones) in naturally aligned 4-byte words: the
- *     up to 3 bytes before an image's first byte and after its last byte
- *     that share such a word with it are read and their values ignored.
- *     Such a word never crosses a page, so any buffer of cudaMalloc or of
- *     a caching allocator qualifies.
+ *     Kernels read image buffers (the inputs of the compress calls, of
+ *     nlc_forward and of the training calls, and the outputs of the decode
+ *     calls, whose decoded pixels are the context of later ones) in naturally
+ *     aligned 4-byte words: the up to 3 bytes before an image's first byte and
+ *     after its last byte that share such a word with it are read and their
+ *     values ignored.  Such a word never crosses a page, so any buffer of
+ *     cudaMalloc or of a caching allocator qualifies.
  *     Container buffers (d_out of the compress calls, d_in of
  *     nlc_decompress) must be 16-byte aligned (NLC_ERR_ARG otherwise).
  *   - Calls taking a `stream` are asynchronous on that stream (NULL = the
@@ -91,8 +91,8 @@ typedef enum {
 
 /* Model configuration: horizon h (1..3), channels C (16, 32, 48 or 64),
  * residual blocks n_res (0..4), mixture components K (1..16), network
- * precision (FP32 SIMT, or BF16 on tcgen05 tensor cores with FP32
- * accumulation).  The mixture, CDF and coder are FP32/integer in both. */
+ * precision (FP32 SIMT, or BF16 on tensor cores with FP32 accumulation).  The
+ * mixture, CDF and coder are FP32/integer in both. */
 typedef struct {
   int32_t h, C, n_res, K, precision;
 } nlc_model_cfg;
