@@ -18,7 +18,6 @@ constexpr int kMq = 65280;              // 2^16 - 256 counts spread by the CDF
 constexpr int kMaxK = 16;               // mixture components
 constexpr int kMaxR = 4;                // residual blocks
 constexpr int kMaxH = 3;                // horizon
-constexpr int kMaxC = 64;               // channels of the local network
 constexpr int kThreads = 256;           // threads of the codec kernels
 constexpr int kWarps = kThreads / 32;
 
@@ -150,12 +149,6 @@ __host__ __device__ __forceinline__ unsigned long long splitmix64_at(unsigned lo
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
   return z ^ (z >> 31);
-}
-__host__ __device__ __forceinline__ uint32_t sample_u16(unsigned long long seed, int image, int y,
-                                                        int x, int c) {
-  const unsigned long long k =
-      ((((unsigned long long)image << 21) + (unsigned long long)y) << 21) + (unsigned long long)x;
-  return (uint32_t)(splitmix64_at(seed, 3ull * k + (unsigned long long)c) >> 48);
 }
 
 // The GPU's global nanosecond timer.

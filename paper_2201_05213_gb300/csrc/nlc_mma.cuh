@@ -160,7 +160,8 @@ __device__ __forceinline__ void mul2(float& a, float& b, float x) {
       : "+f"(a), "+f"(b)
       : "f"(x));
 }
-// ELU of two values (elu_tc's steps) as a BF16 pair.
+// ELU of two values as a BF16 pair: e^x - 1 below zero, by 2^x of the product
+// with log2(e), each step rounded.
 __device__ __forceinline__ uint32_t elu_pair(float x, float y) {
   float a = x, b = y;
   mul2(a, b, 1.4426950408889634f);

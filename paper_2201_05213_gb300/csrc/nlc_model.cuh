@@ -162,12 +162,6 @@ __device__ __forceinline__ float grp_max(float v) {
   return v;
 }
 template <int GW>
-__device__ __forceinline__ float grp_sum(float v) {
-#pragma unroll
-  for (int o = GW / 2; o > 0; o >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o, GW));
-  return v;
-}
-template <int GW>
 __device__ __forceinline__ unsigned grp_mask(int lane) {
   return GW == 32 ? 0xffffffffu : (0xFFFFu << (lane & 16));
 }

@@ -187,10 +187,6 @@ __device__ __forceinline__ void shear_row_features(const uint32_t (&al)[12], int
 // the Ws <= 15 columns before any column are one contiguous byte range.
 constexpr int kRingRowBytes = 96;
 
-__device__ __forceinline__ float elu_tc(float x) {
-  return x > 0.f ? x : __fsub_rn(ex2_approx(__fmul_rn(x, 1.4426950408889634f)), 1.f);
-}
-
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
