@@ -57,12 +57,12 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.41 MB written for
+# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.43 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.62
-TRAFFIC_SRC_SHA = "9e9d2436076cb3d3f22278ad00d44eaefe44ccdd9dd2fd04cc12acbc2e841eb2"
+TRAFFIC_B_PER_PX = 5.64
+TRAFFIC_SRC_SHA = "bc4d7ddde5a64e58926f03d796c5d91cdb775400ba11f54abf01491f24a8a873"
 
 
 # the sources decode_kernel is compiled from
