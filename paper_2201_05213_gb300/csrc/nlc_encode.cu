@@ -131,6 +131,9 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
       if (a.params) {
         const int NO = d.NO;
         const uint32_t wr = wh + (lane & 7) * 16u;
+        // the caller's buffer is an array of floats: pairs of them only where it
+        // starts on 8 bytes (NO and col are even)
+        const bool pairs = (reinterpret_cast<uintptr_t>(a.params) & 7) == 0;
 #pragma unroll 1
         for (int j = 0; 8 * j < NO; j++) {
           uint32_t w[NT8];
@@ -142,10 +145,17 @@ __global__ void __launch_bounds__(32 * kPxWarps, 1) px_bf16_kernel(PxArgs a) {
           if (col < NO) {
             const float2 b = *reinterpret_cast<const float2*>(bh + col);
 #pragma unroll
-            for (int r = 0; r < 2; r++)
-              if (in[r])
-                *reinterpret_cast<float2*>(a.params + out[r] * NO + col) =
-                    make_float2(__fadd_rn(c[2 * r], b.x), __fadd_rn(c[2 * r + 1], b.y));
+            for (int r = 0; r < 2; r++) {
+              if (!in[r]) continue;
+              float* o = a.params + out[r] * NO + col;
+              const float v0 = __fadd_rn(c[2 * r], b.x), v1 = __fadd_rn(c[2 * r + 1], b.y);
+              if (pairs) {
+                *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
+              } else {
+                o[0] = v0;
+                o[1] = v1;
+              }
+            }
           }
         }
       }
