@@ -19,13 +19,6 @@ static int decode_rows(const Dims& d, int n_units, bool win) {
                                                                               : kTileMax / 2;
 }
 
-// The limit is the function's, not a launch's: were it set to each batch's own
-// need, a plan made for a small batch would take it from an earlier plan's
-// larger one.
-static cudaError_t allow_smem(const void* fn) {
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-}
-
 size_t decode_smem_bytes(const Dims& d, int n_units, bool win) {
   return dec_carve(d, n_units, decode_rows(d, n_units, win), win, nullptr);
 }

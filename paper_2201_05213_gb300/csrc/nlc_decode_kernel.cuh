@@ -121,8 +121,6 @@ __device__ __forceinline__ DecShared& dec_shared() {
   return *reinterpret_cast<DecShared*>(dec_smem);
 }
 
-constexpr size_t kMaxSmem = 227 * 1024;
-
 // Carves the shared memory of a tile of `rows` pixels; returns its bytes.
 // win: the sheared model's wavefront decoder.  The whole-warp groups' scratch
 // lies behind the first 16 head-output rows of the BF16 tile region, which a

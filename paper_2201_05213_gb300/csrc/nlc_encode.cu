@@ -304,7 +304,8 @@ static cudaError_t launch_px(const PxArgs& a, int sm_count, cudaStream_t s) {
     threads = kThreads;
     smem = (size_t)f32_plan(d).end * 4 + sizeof(PxSlot) * kF32Rows;
   }
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   PxArgs b = a;
   void* args[] = {&b};

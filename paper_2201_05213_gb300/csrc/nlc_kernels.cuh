@@ -77,6 +77,16 @@ struct CodecBufs {
   unsigned mma_limit = 0;   // timeout is recorded (0: the defaults)
 };
 
+constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory of a CTA
+
+// Lets fn be launched with up to kMaxSmem.  The limit belongs to the function:
+// were it set to each launch's own need, a launch (or plan) of a small batch or
+// model would take it from a larger one made before, or between the limit and
+// the launch of another thread.
+inline cudaError_t allow_smem(const void* fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+}
+
 // Launchers (return cudaError_t of the launch).
 // hash == nullptr: the packed copies only (the content hash is left as is)
 cudaError_t launch_repack(const Dims& d, const float* w, float* simt, uint16_t* umma, float* bias,

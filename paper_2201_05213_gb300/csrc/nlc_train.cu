@@ -8,6 +8,7 @@
 
 #include "nlc_common.cuh"
 #include "nlc_f32.cuh"
+#include "nlc_kernels.cuh"
 #include "nlc_model.cuh"
 #include "nlc_train.cuh"
 
@@ -625,7 +626,7 @@ cudaError_t launch_loss_grad(const Dims& d, const float* wt, const uint8_t* batc
   if (px == 0) return cudaErrorInvalidConfiguration;
   const size_t smem = train_smem_bytes(d, px);
   const void* fn = px == 2 ? loss_grad_fn<2>(d.C) : loss_grad_fn<1>(d.C);
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   float* part_g = reinterpret_cast<float*>(ws);
   float* part_l = part_g + (size_t)g * n_w;

@@ -35,6 +35,7 @@
 
 #include "nlc_common.cuh"
 #include "nlc_mma.cuh"
+#include "nlc_kernels.cuh"
 #include "nlc_model.cuh"
 #include "nlc_tc.cuh"
 #include "nlc_train.cuh"
@@ -776,8 +777,7 @@ cudaError_t launch_tc_train(const Dims& d, const uint16_t* umma, const float* bi
   const long long tiles = (n_px + kTTM - 1) / kTTM;
   const int g = (int)(tiles < sm_count ? (tiles < 1 ? 1 : tiles) : sm_count);
   const void* fn = dparams ? (const void*)tc_train_kernel<1> : (const void*)tc_train_kernel<0>;
-  cudaError_t e =
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.end);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   const int ldw = (n_w + 3) & ~3;
   float* part_g = reinterpret_cast<float*>(ws);
