@@ -69,8 +69,24 @@ __device__ __forceinline__ int slow16() {
   return ((threadIdx.x >> 3) & 3) + 4 * (threadIdx.x >> 6);
 }
 
-// ELU'(t) from u = ELU(t) = e^t - 1 for t <= 0.
-__device__ __forceinline__ float elu_d(float u) { return u > 0.f ? 1.f : __fadd_rn(u, 1.f); }
+// ELU'(x) = e^min(x, 0) from the pre-activation x: ELU(x) + 1 would lose the bits
+// of e^x that the subtraction of 1 rounded away (all of them below -17).  The
+// exponential of a selected argument, because a branch around it took 15 us of
+// a 64 x 32^2 step.
+__device__ __forceinline__ float elu_d(float x) {
+  const float y = x > 0.f ? 0.f : x;
+  return expf(y);
+}
+
+template <int N>
+__device__ __forceinline__ void f32_store(float* p, const float (&v)[N]) {
+  if constexpr (N == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i++) p[i] = v[i];
+  }
+}
 
 __device__ __forceinline__ void red_add(float* p, float v) {
   asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
@@ -324,12 +340,16 @@ __device__ float pixel_nll_grad(const float* P, int K, const int (&v)[3], float 
 // stream and of its gradient in registers; a layer costs one barrier.
 // Measured, 64 x 32^2 (h = 3, C = 64, R = 2, K = 10): 1424 us with 64-pixel tiles and
 // weights read through L2, 505 us so (FMA pipe about a third busy; the rest is
-// latency at two warps per scheduler).
+// latency at two warps per scheduler).  The pre-activations, which the adjoint
+// needs for ELU', do not fit in shared memory beside the activations (46 KB):
+// they pass through the workspace (40 KB per CTA, in L2), and their reads and
+// exponentials take the call from 521 to 541 us.
 template <int NB, int PX>
 __global__ void __launch_bounds__(kThreads, 1)
     loss_grad_kernel(Dims d, const float* __restrict__ wt, const uint8_t* __restrict__ batch,
                      int N, int H, int W, const float* __restrict__ dparams,
-                     float* __restrict__ part_g, float* __restrict__ part_l, int n_w) {
+                     float* __restrict__ part_g, float* __restrict__ part_l, int n_w,
+                     float* pre_act) {
   extern __shared__ __align__(16) float sm[];
   constexpr int kTM = tile_px<PX>(), kTLd = tile_ld<PX>();
   const TrainPlan pl = train_plan(d, PX);
@@ -369,6 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const long long HW = (long long)H * W, n_px = (long long)N * HW;
   const float scale = 1.f / (0.6931471805599453f * 3.f * (float)n_px);
   const long long ntiles = (n_px + kTM - 1) / kTM;
+  // the CTA's pre-activations [2R + 1][C][kTM], written and read by this CTA only
+  float* Z = pre_act + (size_t)blockIdx.x * (2 * R + 1) * C * kTM;
   // forward: pixels PX fm .. (neighbouring lanes) of outputs NB fg ..;
   // adjoint: the same pixels of mg, outputs g + 16 j (neighbouring lanes)
   const int fm = threadIdx.x & 15, fg = threadIdx.x >> 4;
@@ -411,12 +433,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       float res[NB][PX];
       const float* bias = sm + pl.bias + NB * fg;
       float* U = sm + pl.U + NB * fg * kTLd + PX * fm;  // the thread's block of the next tile
+      float* z = Z + NB * fg * kTM + PX * fm;
       auto store = [&](const float (&v)[NB][PX]) {
 #pragma unroll
-        for (int b = 0; b < NB; b++)
+        for (int b = 0; b < NB; b++) {
+          f32_store<PX>(z + b * kTM, v[b]);
 #pragma unroll
           for (int a = 0; a < PX; a++) U[b * kTLd + a] = elu_f(v[b][a]);
+        }
         U += C * kTLd;
+        z += C * kTM;
         bias += C;
       };
       f32_dot<PX, NB>(sm + pl.X + PX * fm, kTLd, F, sm + pl.w0 + NB * fg, ldc, res);
@@ -479,14 +505,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     float da[NB][PX], acc[NB][PX];
     float* G = sm + pl.G;
     float* G2 = sm + pl.G2;
-    // gradient through ELU of the thread's block of activations U
-    auto through = [&](const float* U, float (&v)[NB][PX]) {
+    // gradient through ELU of the thread's block of layer l
+    auto through = [&](int l, float (&v)[NB][PX]) {
+      const float* z = Z + (l * C + g) * kTM + PX * mg;
 #pragma unroll
       for (int j = 0; j < NB; j++) {
-        float u[PX];
-        f32_load<PX>(U + (g + 16 * j) * kTLd + PX * mg, u);
+        float x[PX];
+        f32_load<PX>(z + 16 * j * kTM, x);
 #pragma unroll
-        for (int a = 0; a < PX; a++) v[j][a] = __fmul_rn(v[j][a], elu_d(u[a]));
+        for (int a = 0; a < PX; a++) v[j][a] = __fmul_rn(v[j][a], elu_d(x[a]));
       }
     };
     auto put = [&](float* o, const float (&v)[NB][PX]) {
@@ -496,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int a = 0; a < PX; a++) o[(g + 16 * j) * kTLd + PX * mg + a] = v[j][a];
     };
     input_grad<PX, NB>(sm + pl.wh, ldh, sm + pl.DP, NO, da);  // WH^T dP
-    through(Ul, da);
+    through(2 * R, da);
     put(G, da);  // P is dead: the likelihood has read it
     for (int n = 0; n < NO; n += 16 * 4) {  // 16 x 4 outputs a round, the last as many as needed
       if (NO - n > 48) weight_grad<PX, 4, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
@@ -509,13 +536,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       const size_t oW2 = ob1 + C, ob2 = oW2 + (size_t)C * C;
       const float* V = sm + pl.U + (2 * r + 1) * C * kTLd;
       input_grad<PX, NB>(sm + pl.w1 + (2 * r + 1) * pl.wstride, ldc, G, C, acc);  // dv = W2^T da
-      through(V, acc);
+      through(2 * r + 1, acc);
       put(G2, acc);
       weight_grad<PX, NB, NB>(G, C, V, C, gW + oW2, gW + ob2);
       __syncthreads();
       const float* Ur = V - C * kTLd;
       input_grad<PX, NB>(sm + pl.w1 + 2 * r * pl.wstride, ldc, G2, C, acc);  // du = W1^T dz
-      through(Ur, acc);
+      through(2 * r, acc);
 #pragma unroll
       for (int j = 0; j < NB; j++)
 #pragma unroll
@@ -602,7 +629,8 @@ size_t train_ws_bytes(const Dims& d, long long n_px, int sm_count) {
   const size_t nw = (size_t)d.C * d.F + d.C + (size_t)d.R * (2 * d.C * d.C + 2 * d.C) +
                     (size_t)d.NO * d.C + d.NO;
   const int g = train_grid(d, n_px, sm_count);
-  return ((size_t)g * nw + g + 64) * 4;
+  const size_t pre = (size_t)(2 * d.R + 1) * d.C * kTG * train_px(d);  // pre-activations
+  return ((size_t)g * (nw + 1 + pre) + 64) * 4;
 }
 
 template <int PX>
@@ -630,9 +658,11 @@ cudaError_t launch_loss_grad(const Dims& d, const float* wt, const uint8_t* batc
   if (e != cudaSuccess) return e;
   float* part_g = reinterpret_cast<float*>(ws);
   float* part_l = part_g + (size_t)g * n_w;
+  // behind the slots and losses, on 256 bytes
+  float* pre_act = part_g + (((size_t)g * (n_w + 1) + 63) & ~(size_t)63);
   Dims dd = d;
   int nw = n_w;
-  void* args[] = {&dd, &wt, &batch, &N, &H, &W, &dparams, &part_g, &part_l, &nw};
+  void* args[] = {&dd, &wt, &batch, &N, &H, &W, &dparams, &part_g, &part_l, &nw, &pre_act};
   if ((e = cudaLaunchKernel(fn, dim3(g), dim3(kThreads), args, smem, s)) != cudaSuccess) return e;
   return launch_reduce_grad(part_g, dparams ? nullptr : part_l, g, n_w, n_w, n_px, grad, loss, s);
 }
