@@ -495,9 +495,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint8_t* px = batch + ((long long)s.x * HW + (long long)s.y * W + s.z) * 3;
         v[0] = px[0], v[1] = px[1], v[2] = px[2];
       }
-      const float nll = pixel_nll_grad(sm + pl.P + m * pl.ldp, K, v, s.x >= 0 ? scale : 0.f,
-                                       sm + pl.DP + m, kTLd, l);
-      if (l == 0 && s.x >= 0) loss = __fadd_rn(loss, nll);
+      const float nll = pixel_nll_grad(sm + pl.P + m * pl.ldp, K, v, scale, sm + pl.DP + m, kTLd, l);
+      if (s.x < 0) {  // its terms may be infinite: not multiplied by 0 but left out
+        __syncwarp(0xffu << (threadIdx.x & 24));
+        for (int k = l; k < NO; k += kLanes) sm[pl.DP + k * kTLd + m] = 0.f;
+      } else if (l == 0) {
+        loss = __fadd_rn(loss, nll);
+      }
     }
     __syncthreads();
     // ---- adjoint ----
