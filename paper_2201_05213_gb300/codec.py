@@ -160,6 +160,8 @@ class DecodePlan:
 
 
 def _batch_images(batch):
+    if batch.shape[0] == 0:
+        raise IndexError("a batch without images")
     return N._batch(batch) if batch.is_contiguous() else N._images(list(batch))
 
 
