@@ -88,8 +88,29 @@ __device__ __forceinline__ void f32_store(float* p, const float (&v)[N]) {
   }
 }
 
-__device__ __forceinline__ void red_add(float* p, float v) {
-  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+// weight_grad of a thread that has had tiny sums (from then on: a zero would
+// flush them): the same sums, one after another.  Asking for it takes a call
+// without tiny sums from 543 to 551 us (64 x 32^2), because no reduction starts
+// before the last sum is known; the choice at each of the unrolled sums takes
+// it to 554-580.
+template <int PX>
+__device__ __noinline__ void weight_grad_tiny(const float* G, int Nn, const float* X, int Kk,
+                                              float* __restrict__ gW, float* __restrict__ gb,
+                                              int n0, int NB, int KB) {
+  constexpr int kTM = tile_px<PX>(), kTLd = tile_ld<PX>();
+  const int kg = fast16();
+  for (int n = n0; n < Nn && n < n0 + 16 * NB; n += 16) {
+    for (int k = kg; k < Kk && k < kg + 16 * KB; k += 16) {
+      float acc = 0.f;
+      for (int m = 0; m < kTM; m++) acc = __fmaf_rn(G[n * kTLd + m], X[k * kTLd + m], acc);
+      slot_add(gW + (size_t)n * Kk + k, acc);
+    }
+    if (kg == 0) {
+      float bs = 0.f;
+      for (int m = 0; m < kTM; m++) bs = __fadd_rn(bs, G[n * kTLd + m]);
+      slot_add(gb + n, bs);
+    }
+  }
 }
 
 // Weight gradient of one layer: gW[n][k] += sum_m G[n][m] X[k][m] for n < Nn,
@@ -101,7 +122,7 @@ __device__ __forceinline__ void red_add(float* p, float v) {
 // fixed, and no thread waits for the old value (reading it back cost 119 of
 // 626 us per 64 x 32^2 step).
 template <int PX, int NB, int KB>
-__device__ __forceinline__ void weight_grad(const float* G, int Nn, const float* X, int Kk,
+__device__ __forceinline__ void weight_grad(bool& tiny, const float* G, int Nn, const float* X, int Kk,
                                             float* __restrict__ gW, float* __restrict__ gb,
                                             int first = 0) {
   constexpr int kTM = tile_px<PX>(), kTLd = tile_ld<PX>();
@@ -150,6 +171,21 @@ __device__ __forceinline__ void weight_grad(const float* G, int Nn, const float*
     if (m + 8 < kTM) load(0, m + 8);
     fma(1);
   }
+  // smallest magnitude but 0, as twice the bits less 1 (a chain per output)
+  unsigned lo[NB];
+#pragma unroll
+  for (int b = 0; b < NB; b++) {
+    lo[b] = 2u * __float_as_uint(bs[b]) - 1u;
+#pragma unroll
+    for (int j = 0; j < KB; j++) lo[b] = min(lo[b], 2u * __float_as_uint(acc[b][j]) - 1u);
+  }
+#pragma unroll
+  for (int b = 1; b < NB; b++) lo[0] = min(lo[0], lo[b]);
+  tiny |= lo[0] < 2u * __float_as_uint(kSlotTiny) - 1u;
+  if (tiny) {
+    weight_grad_tiny<PX>(G, Nn, X, Kk, gW, gb, n0, NB, KB);
+    return;
+  }
 #pragma unroll
   for (int b = 0; b < NB; b++) {
     const int n = n0 + 16 * b;
@@ -157,9 +193,9 @@ __device__ __forceinline__ void weight_grad(const float* G, int Nn, const float*
 #pragma unroll
     for (int j = 0; j < KB; j++) {
       const int k = kg + 16 * j;
-      if (k < Kk) red_add(gW + (size_t)n * Kk + k, acc[b][j]);
+      if (k < Kk) slot_red(gW + (size_t)n * Kk + k, acc[b][j]);
     }
-    if (kg == 0) red_add(gb + n, bs[b]);
+    if (kg == 0) slot_red(gb + n, bs[b]);
   }
 }
 
@@ -396,6 +432,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int fm = threadIdx.x & 15, fg = threadIdx.x >> 4;
   const int g = fast16(), mg = slow16();
   float loss = 0.f;
+  bool tiny = false;  // a sum below kSlotTiny is in the thread's part of the slot
   for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     if (threadIdx.x < kTM) {
       const long long q = tile * kTM + threadIdx.x;
@@ -530,9 +567,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     through(2 * R, da);
     put(G, da);  // P is dead: the likelihood has read it
     for (int n = 0; n < NO; n += 16 * 4) {  // 16 x 4 outputs a round, the last as many as needed
-      if (NO - n > 48) weight_grad<PX, 4, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
-      else if (NO - n > 16) weight_grad<PX, 3, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
-      else weight_grad<PX, 1, NB>(sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+      if (NO - n > 48) weight_grad<PX, 4, NB>(tiny, sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+      else if (NO - n > 16) weight_grad<PX, 3, NB>(tiny, sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
+      else weight_grad<PX, 1, NB>(tiny, sm + pl.DP, NO, Ul, C, gW + oWH, gW + obH, n);
     }
     __syncthreads();
     for (int r = R - 1; r >= 0; r--) {
@@ -542,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       input_grad<PX, NB>(sm + pl.w1 + (2 * r + 1) * pl.wstride, ldc, G, C, acc);  // dv = W2^T da
       through(2 * r + 1, acc);
       put(G2, acc);
-      weight_grad<PX, NB, NB>(G, C, V, C, gW + oW2, gW + ob2);
+      weight_grad<PX, NB, NB>(tiny, G, C, V, C, gW + oW2, gW + ob2);
       __syncthreads();
       const float* Ur = V - C * kTLd;
       input_grad<PX, NB>(sm + pl.w1 + 2 * r * pl.wstride, ldc, G2, C, acc);  // du = W1^T dz
@@ -552,13 +589,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int a = 0; a < PX; a++) da[j][a] = __fadd_rn(da[j][a], acc[j][a]);
       put(G, da);
-      weight_grad<PX, NB, NB>(G2, C, Ur, C, gW + oW1, gW + ob1);
+      weight_grad<PX, NB, NB>(tiny, G2, C, Ur, C, gW + oW1, gW + ob1);
       __syncthreads();
     }
     switch ((F + 15) / 16) {
-      case 1: weight_grad<PX, NB, 1>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
-      case 3: weight_grad<PX, NB, 3>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
-      default: weight_grad<PX, NB, 5>(G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+      case 1: weight_grad<PX, NB, 1>(tiny, G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+      case 3: weight_grad<PX, NB, 3>(tiny, G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
+      default: weight_grad<PX, NB, 5>(tiny, G, C, sm + pl.X, F, gW + oW0, gW + ob0); break;
     }
     __syncthreads();
   }

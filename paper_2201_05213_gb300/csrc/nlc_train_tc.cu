@@ -214,14 +214,6 @@ __device__ __noinline__ void tt_gather(const Dims& d, const uint8_t* px0, int W,
                     reinterpret_cast<uint16_t*>(X) + (m >> 3) * (d.Fp >> 3) * 64 + (m & 7) * 8, 64);
 }
 
-__device__ __forceinline__ void red_add2(float* p, float a, float b) {
-  asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b)
-               : "memory");
-}
-__device__ __forceinline__ void red_add1(float* p, float a) {
-  asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory");
-}
-
 // 16 rows x 8 FP32 columns of tensor memory, without waiting: lane l gets
 // columns 2 (l % 4), + 1 of rows l / 4 (r[0], r[1]) and l / 4 + 8 (r[2], r[3]).
 __device__ __forceinline__ void tmem_ld16x8_nw(uint32_t taddr, uint32_t (&r)[4]) {
@@ -258,9 +250,16 @@ __device__ __noinline__ void tt_flush(uint32_t tmem, int buf, int n_out, int n_i
     float* p = gW + (size_t)o * ld + col;
     if (col < n_in) {
       auto put = [&](int k, uint32_t x, uint32_t y) {  // row o + 8 k
-        if (o + 8 * k < n_out)
-          red_add2(p + (size_t)(8 * k) * ld, __fmul_rn(__uint_as_float(x), scale),
-                   __fmul_rn(__uint_as_float(y), scale));
+        if (o + 8 * k >= n_out) return;
+        float* w = p + (size_t)(8 * k) * ld;
+        const float a = __fmul_rn(__uint_as_float(x), scale);
+        const float b = __fmul_rn(__uint_as_float(y), scale);
+        if (fminf(fabsf(a), fabsf(b)) >= kSlotTiny) {
+          slot_red2(w, a, b);
+        } else {
+          slot_add(w, a);
+          slot_add(w + 1, b);
+        }
       };
       put(0, r0[0], r0[1]);
       put(1, r0[2], r0[3]);
@@ -277,7 +276,7 @@ __device__ __noinline__ void tt_flush(uint32_t tmem, int buf, int n_out, int n_i
                  : "memory");
     tmem_wait_ld();
     asm volatile("" : "+r"(rb));
-    if (32 * q + lane < n_out) red_add1(gb + 32 * q + lane, __uint_as_float(rb));
+    if (32 * q + lane < n_out) slot_add(gb + 32 * q + lane, __uint_as_float(rb));
   }
 }
 
