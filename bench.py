@@ -57,12 +57,12 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.44 MB written for
+# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.25 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.64
-TRAFFIC_SRC_SHA = "8000785cdbba04239ea44ca579f185c1bc7a9109e402b45b1fef4f6b5ef65186"
+TRAFFIC_B_PER_PX = 5.46
+TRAFFIC_SRC_SHA = "af0123a0c137134fc167ffd7801420057d207ae7fad39318f607858cd69526c9"
 
 
 # the sources decode_kernel is compiled from

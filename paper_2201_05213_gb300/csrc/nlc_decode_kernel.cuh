@@ -49,13 +49,13 @@ __host__ __device__ constexpr int decode_threads() { return PREC == PREC_BF16 ? 
 struct alignas(16) DecUnit {
   uint8_t* px;      // first pixel
   int Hu, Wu;       // size
-  int row_bytes;    // row stride of the image
+  uint32_t row_bytes;  // row stride of the image (two rows of 2^30 pixels fit)
   int stream_base;  // first rANS stream
   int start_step;   // step of its first pixel
   int ring_row;     // first row in the sheared rings
 };
 __device__ __forceinline__ DecUnit dec_unit(const Unit& u) {
-  return DecUnit{u.img + ((long long)u.y0 * u.img_W + u.x0) * 3, u.Hu, u.Wu, 3 * u.img_W,
+  return DecUnit{u.img + ((long long)u.y0 * u.img_W + u.x0) * 3, u.Hu, u.Wu, 3u * u.img_W,
                  u.stream_base, u.start_step, u.ring_row};
 }
 
@@ -486,7 +486,7 @@ __device__ __forceinline__ void sched_slots(int step, int base, int n, int nt) {
       ps.i = tau / U.Wu;
       ps.j = tau - ps.i * U.Wu;
     }
-    ps.px = U.px + (long long)ps.i * U.row_bytes + 3 * ps.j;
+    ps.px = U.px + (long long)ps.i * U.row_bytes + 3LL * ps.j;
     ps.Wu = U.Wu;
     ps.row_bytes = U.row_bytes;
     ps.stream = U.stream_base + (layout == 1 ? ps.i : 0);

@@ -433,7 +433,7 @@ struct alignas(16) DecSlot {
   uint8_t* px;    // its address in the image
   int i, j;       // position inside its unit
   int Wu;         // width of the unit
-  int row_bytes;  // row stride of the image
+  uint32_t row_bytes;  // row stride of the image
   int stream;     // its rANS stream
   int unit;       // unit index; bit 31: the stream's last pixel
 };

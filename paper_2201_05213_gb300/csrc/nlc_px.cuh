@@ -28,7 +28,7 @@ struct alignas(16) PxSlot {
   const uint8_t* px;  // its address in the image
   int i, j;           // position inside its unit
   int Wu;             // width of the unit
-  int row_bytes;      // row stride of the image
+  uint32_t row_bytes;  // row stride of the image (two rows of 2^30 pixels fit)
   long long out;      // forward: index of its outputs (images in order, raster)
 };
 
@@ -73,7 +73,7 @@ __device__ __forceinline__ int px_slots(const Unit* __restrict__ units, int n_un
     const long long row = U.y0 + s.i;
     s.px = U.img + (row * U.img_W + (U.x0 + s.j)) * 3;
     s.Wu = U.Wu;
-    s.row_bytes = 3 * U.img_W;
+    s.row_bytes = 3u * U.img_W;
     s.out = U.img_px_base + row * U.img_W + (U.x0 + s.j);
     slots[lane] = s;
     hint = u;
