@@ -57,12 +57,12 @@ def workload_name():
 
 
 # DRAM traffic of decode_kernel per decoded pixel from one ncu capture of the
-# small case at 16 CTAs (1x1024^2: 5.48 MB read + 0.25 MB written for
+# small case at 16 CTAs (1x1024^2: 5.82 MB read + 0.28 MB written for
 # 1,048,576 px), scaled to a launch by its pixels.  It holds only for the
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
-TRAFFIC_B_PER_PX = 5.46
-TRAFFIC_SRC_SHA = "af0123a0c137134fc167ffd7801420057d207ae7fad39318f607858cd69526c9"
+TRAFFIC_B_PER_PX = 5.81
+TRAFFIC_SRC_SHA = "a628a5c49c4d148fb7168b62a52521d3104558141f206a8f6de375a1c8be9074"
 
 
 # the sources decode_kernel is compiled from

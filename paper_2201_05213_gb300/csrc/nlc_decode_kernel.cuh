@@ -92,12 +92,11 @@ struct DecSmem {
   int prow;   // sheared wavefront decoder: output row of the tile's pixel s
   int rofs;   // sheared wavefront decoder: ring byte offset of the tile's pixel s
   int wrow;   // sheared wavefront decoder: (unit, unit row) of window row rho
-  int sh;     // 33 long long: the schedule's warp sums (ints)
-  int share;  // int2 [kShares], behind the warp sums: shares [x, y) of a step and of the next one
+  int sh;     // 64 ints: the schedule's warp sums
   int pc;     // 16 profiling accumulators (thread 0 only)
   int units;  // DecUnit: the batch's units, where they fit (else 0: read from global memory)
   int pre;    // front prefix of the units
-  int flag;   // [0] stop, [1..3] sheared tile, [4], [5] units of the share
+  int flag;   // [0] stop, [1..3] sheared tile, [4], [5] units of the share, [6..9] shares (share_at)
 };
 
 // Copies of the CTA's share, by the step's parity.  Every warp reads its copy
@@ -159,10 +158,9 @@ __host__ __device__ inline size_t dec_carve(const Dims& d, int n_pre, int rows, 
     z.prow = take(sizeof(int) * rows);
     z.rofs = take(sizeof(int) * rows);
   }
-  z.sh = take(sizeof(long long) * 33);
-  z.share = z.sh + (int)sizeof(int) * 16;
+  z.sh = take(sizeof(int) * 64);
   z.pc = take(sizeof(long long) * 16);
-  z.flag = take(sizeof(int) * 6);
+  z.flag = take(sizeof(int) * (6 + 2 * kShares));
   z.pre = take(sizeof(int) * ((size_t)n_pre + 1));
   if (kSharedHead + off + sizeof(DecUnit) * (size_t)n_pre <= kMaxSmem)
     z.units = take(sizeof(DecUnit) * (size_t)n_pre);
@@ -358,14 +356,14 @@ __device__ __forceinline__ int2 sched_share(int F) {
   return make_int2(lo, lo + (int)each + (blockIdx.x < more ? 1 : 0));
 }
 
-// The record of step's share.
-__device__ __forceinline__ int2& share_at(int step) {
-  return dec_at<int2>(dec_shared().t.share)[(unsigned)step % kShares];
+// The CTA's share [x, y) of a step's pixels, beside the flags.
+__device__ __forceinline__ int2& share_at(int* flag, int step) {
+  return reinterpret_cast<int2*>(flag + 6)[(unsigned)step % kShares];
 }
 
 // Fronts of all units: pre[u] = exclusive prefix of the front sizes,
 // pre[n_units] = their total F; flag[4], flag[5] = the units that hold the
-// first and the last pixel of this CTA's share share_at(step).
+// first and the last pixel of this CTA's share.
 //
 // Up to kWarpUnits units, every warp computes all of it (and stores the same
 // values): one or two warp scans cost less than the two barriers that a scan
@@ -400,7 +398,7 @@ static __device__ __forceinline__ void sched_front_warp(int step) {
   put(lane + 32, F0 + x1 - c1, c1);
   if (lane == 0) {
     pre[n_units] = F;
-    share_at(step) = sh;
+    share_at(flag, step) = sh;
   }
   __syncwarp();
 }
@@ -450,7 +448,7 @@ static __device__ __forceinline__ void sched_front(int step, int nt) {
   }
   if (threadIdx.x == 0) {
     pre[n_units] = F;
-    share_at(step) = share;
+    share_at(flag, step) = share;
   }
   part_sync(nt);
 }
@@ -594,7 +592,7 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
   constexpr int NS = NT - 32;
   sched_front(0, NT);
   tick(0);
-  int lo = share_at(0).x, hi = share_at(0).y;  // the CTA's share of the step's pixels
+  int lo = share_at(flag, 0).x, hi = share_at(flag, 0).y;  // the CTA's share of the step's pixels
   if (lo < hi) sched_slots<SHEAR>(0, lo, min(rows, hi - lo), NT);
   __syncthreads();
   tick(1);
@@ -678,8 +676,8 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
     } else {
       sched_front(step + 1, NS);
       tick(0);
-      lo = share_at(step + 1).x;
-      hi = share_at(step + 1).y;
+      lo = share_at(flag, step + 1).x;
+      hi = share_at(flag, step + 1).y;
       if (lo < hi) sched_slots<SHEAR>(step + 1, lo, min(rows, hi - lo), NS);
       tick(1);
     }
@@ -688,8 +686,8 @@ __global__ void __launch_bounds__(decode_threads<PREC>(), 1) decode_kernel(Decod
     } else {
       __syncthreads();
     }
-    lo = share_at(step + 1).x;
-    hi = share_at(step + 1).y;
+    lo = share_at(flag, step + 1).x;
+    hi = share_at(flag, step + 1).y;
     tick(4);
     if (stamp && blockIdx.x == 0 && step + 1 < a.n_times) a.times[step + 1] = global_ns();
   }
