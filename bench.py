@@ -62,7 +62,7 @@ def workload_name():
 # kernel sources it was taken on: TRAFFIC_SRC_SHA is the sha256 of
 # DECODER_SOURCES, and any other sources report null.
 TRAFFIC_B_PER_PX = 5.81
-TRAFFIC_SRC_SHA = "a628a5c49c4d148fb7168b62a52521d3104558141f206a8f6de375a1c8be9074"
+TRAFFIC_SRC_SHA = "4c8d92baad15a11d88950a7a809ab88ce0bd60020e8e9c9bd0ef65801ca9109f"
 
 
 # the sources decode_kernel is compiled from

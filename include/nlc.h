@@ -149,15 +149,15 @@ int nlc_sync_status(nlc_ctx* ctx, nlc_stream stream);
 int nlc_set_tuning(nlc_ctx* ctx, int px_per_cta, int max_ctas);
 
 /* Limits of the decoder's bounded waits (also the sampler's): polls of the
- * grid barrier between wavefront steps and, in the BF16 network, of the
- * exchange between two layers' MMAs before the wait gives up (0 = the
- * defaults, 2^25 and 2^22 polls, far beyond any normal wait).  A wait that
- * gives up records NLC_ERR_TIMEOUT in the context's status and releases every
- * CTA of the launch, which leaves the decode loop (an exchange first waits,
- * bounded, for the warps it shares the layer with); the context stays usable.
- * Small limits exist to exercise that path: a reduced MMA limit counts
- * non-blocking tests of the exchange, which without one is a hardware barrier
- * of the warps involved. */
+ * grid barrier between wavefront steps (0 = the default, 2^25, far beyond any
+ * normal wait) and of the exchange between two layers of the BF16 network.
+ * The exchange is a hardware barrier of the warps that share the layer, which
+ * counts no polls, at mma_polls = 0 and from 2^22 up; a smaller limit runs it
+ * through an mbarrier and counts non-blocking tests of it.  A wait that gives
+ * up records NLC_ERR_TIMEOUT in the context's status and releases every CTA of
+ * the launch, which leaves the decode loop (an exchange first waits, bounded,
+ * for the warps it shares the layer with); the context stays usable.  Small
+ * limits exist to exercise that path. */
 int nlc_set_wait_limits(nlc_ctx* ctx, uint32_t grid_polls, uint32_t mma_polls);
 
 /* Decoder phase profile (per-step latency against the dependency-bound step

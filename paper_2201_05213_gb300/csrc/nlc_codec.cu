@@ -235,7 +235,10 @@ cudaError_t launch_hash(const Dims& d, const float* w, int n_w, unsigned long lo
 // streams than the SMs have warps a warp each shortens it (one stream of 3,072
 // symbols: 502 us by a thread that divides and waits for each symbol, 259 us by
 // a warp); with more, threads keep all lanes busy (49 k streams of 768 symbols:
-// 442 us before, 412 us now).
+// 442 us before, 412 us now).  Streams of 768 symbols, by warps and by threads:
+// 72 and 173 us at 4 streams per SM, 88 / 174 at 16, 113 / 175 at 24, 149 / 175
+// at 32, 206 / 176 at 48; of 192 symbols 40 / 47 us at 32 and 55 / 47 at 48, of
+// 3,072 582 / 694 and 811 / 693: they cross at about 38 streams per SM.
 template <bool WARP>
 __global__ void rans_enc_kernel(const Unit* __restrict__ units, int n_units, int n_streams,
                                 int layout, const uint32_t* __restrict__ stage,

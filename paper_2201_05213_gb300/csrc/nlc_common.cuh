@@ -233,9 +233,7 @@ __device__ __forceinline__ bool grid_wait(unsigned* count, unsigned nblocks, uns
   return *s_flag == 0;
 }
 
-// Front of a unit at its local step tau.
-//   wavefront (Section 3): rows i with j = tau - (h+1) i in [0, Wu)
-//   raster: the single pixel tau of the unit in raster order.
+// A unit's pixels of one step.
 struct Front {
   int i_lo, n;  // first row and number of pixels
 };

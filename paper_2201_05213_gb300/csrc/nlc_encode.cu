@@ -6,9 +6,9 @@
 
 namespace nlc {
 
-// Warps per CTA of the BF16 kernel.  Four per scheduler at 128 registers (16
-// to 24 bytes spilled) hide the chains better than three at 168: 5.5 against
-// 6.1 ms for 12.6 M pixels; 14 leave the schedulers uneven (6.3 ms).
+// Warps per CTA of the BF16 kernel.  Four per scheduler at 128 registers (up to
+// 32 bytes spilled) hide the chains better than three at 168: 4.9 against 5.3 ms
+// for the tables of 12.6 M pixels; 14 leave the schedulers uneven (5.6 ms).
 constexpr int kPxWarps = 16;
 
 struct PxArgs {

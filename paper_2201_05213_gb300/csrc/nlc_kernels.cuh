@@ -73,8 +73,8 @@ struct CodecBufs {
   unsigned long long* prof = nullptr;  // decoder phase cycle counters (16), optional
   unsigned long long* times = nullptr;  // decoder step end times, optional
   long long n_times = 0;
-  unsigned spin_limit = 0;  // decoder: polls of the grid barrier / an MMA completion before a
-  unsigned mma_limit = 0;   // timeout is recorded (0: the defaults)
+  unsigned spin_limit = 0;  // decoder: polls of the grid barrier / of a layer's exchange before
+  unsigned mma_limit = 0;   // a timeout is recorded (0: the defaults)
 };
 
 constexpr size_t kMaxSmem = 227 * 1024;  // dynamic shared memory of a CTA

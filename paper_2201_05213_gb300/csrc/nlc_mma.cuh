@@ -533,7 +533,9 @@ __device__ __forceinline__ void gather_row_shear(const Slot& s, int dd, int h, i
 // Columns 2 part, 2 part + 1 of one context row (masked tile): the same
 // features from the two or three words around their six bytes, for tiles of so
 // few pixels that a lane per row would leave most warps idle (8 pixels: one
-// warp with 250 instructions, 1.08 us; so 0.79).
+// warp with 250 instructions, 1.08 us; so 0.79).  A whole step: 7.30 against
+// 7.61 us at 8 pixels, 8.09 / 8.28 at 16, 10.28 / 10.42 at 24, 10.37 / 10.41 at
+// 32, where the two meet and the CTA's warps are all in use.
 template <class Slot>
 __device__ __forceinline__ void gather_part(const Slot& s, int r, int part, int h, int F, int Fp,
                                             uint16_t* X, int cs) {

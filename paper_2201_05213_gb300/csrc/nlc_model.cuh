@@ -112,14 +112,15 @@ __device__ __forceinline__ float log_bin_mass_f(float m, float inv, float lme, i
   return __fadd_rn(__fsub_rn(-softplus_f(-a), softplus_f(b)), lme);
 }
 
-// Scratch of one coding group (a warp, or half a warp) in the CDF stage:
+// Scratch of one coding group in the CDF stage (a warp in the decoder, half a
+// warp in the table entry point):
 // the channel's active components (weight >= kWmin), compacted in
 // increasing component order, as (m_k, c_k = log2(e)/s_k, w_k 2^23, 0),
 // then zero entries (weight 0, term 0) up to 2 kMaxK, so that unrolled
 // loops may read past the last active component.
 struct alignas(16) WarpScratch {
   float4 cp[2 * kMaxK];
-  float4 pad;  // 528-byte stride: the two groups of a warp read different banks
+  float4 pad;  // 528-byte stride: two half-warp groups read different banks
 };
 
 // Table of one coding warp for decoding with an explicit cum[0..255]
@@ -285,8 +286,8 @@ __device__ __forceinline__ float comp_mean(const CompState& cs, int ch, int r, i
 // back from its bits.  kClamp clamps z to [-126, 126] first, which changes no
 // term: past 126 the term is 0 and below -126 it is rint(w) either way
 // (1 + 2^z rounds to 1).  The whole-warp search, one pixel per warp and bound
-// by latency, measured faster with the clamp; the 16-lane search, bound by
-// throughput, without it.
+// by latency, measured faster with the clamp; the quads, bound by instruction
+// issue, go without it.
 template <bool kClamp = false>
 __device__ __forceinline__ uint32_t cdf_term(float e, const float4& p) {
   float z = __fmul_rn(__fsub_rn(p.x, e), p.y);

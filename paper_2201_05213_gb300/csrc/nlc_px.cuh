@@ -8,11 +8,11 @@
 // head's weight rows are read in an order that leaves every lane with whole
 // mixture components of its two pixels, so the coding starts from registers
 // too.  Only the context tile (16 pixels) passes through shared memory, where
-// the weights stay for the CTA's lifetime.  Bound: instruction issue (57 %
-// of the slots at twelve warps, 310 warp instructions per pixel; MUFU 25 %,
-// tensor pipe 21 %).  Measured, the tables of 12.6 M pixels (h = 3, C = 64, R
-// = 2, K = 10): 18.6 ms with one 128-pixel tcgen05 tile at a time per SM and 16
-// lanes per pixel, 4.8 ms so.
+// the weights stay for the CTA's lifetime.  Bound: instruction issue (1024^2
+// pixels: 63 % of the slots at sixteen warps, 284 warp instructions per pixel;
+// MUFU 22 %, tensor pipe 26 %).  Measured, the tables of 12.6 M pixels (h = 3, C
+// = 64, R = 2, K = 10): 18.6 ms with one 128-pixel tcgen05 tile at a time per SM
+// and 16 lanes per pixel, 4.9 ms so.
 #pragma once
 
 #include "nlc_mma.cuh"

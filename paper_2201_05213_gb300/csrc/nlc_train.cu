@@ -379,7 +379,8 @@ __device__ float pixel_nll_grad(const float* P, int K, const int (&v)[3], float 
 // latency at two warps per scheduler).  The pre-activations, which the adjoint
 // needs for ELU', do not fit in shared memory beside the activations (46 KB):
 // they pass through the workspace (40 KB per CTA, in L2), and their reads and
-// exponentials take the call from 521 to 541 us.
+// exponentials take the call (kernel and reduction) from 521 to 543 us; the
+// small sums of weight_grad take it to 551.
 template <int NB, int PX>
 __global__ void __launch_bounds__(kThreads, 1)
     loss_grad_kernel(Dims d, const float* __restrict__ wt, const uint8_t* __restrict__ batch,

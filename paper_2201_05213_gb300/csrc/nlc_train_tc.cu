@@ -535,7 +535,8 @@ __device__ __noinline__ float tt_likelihood(const Dims& d, uint32_t tcol, const 
 // per CTA) spends 51 us in the likelihood, 42 and 38 in the forward and
 // backward epilogues, 35 in the flushes, 24 in the weight-gradient chains.
 // 287 us with 256 threads, the slot read back in every flush and the context
-// gathered twice; 190 us so.
+// gathered twice; 190 us so (a call with its reduction 196 us, 201 with the test
+// for small sums).
 //
 // MODE 0: dP = gradient of the mean code length in bits per dimension of the
 // batch (Eq. 2), the loss summed per CTA into part_l; MODE 1: dP = the given
